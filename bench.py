@@ -54,8 +54,15 @@ OPS_PER_DATA_SPAXEL = 10
 # three FMAs (s0 += w q0, s1 += w l1, s2 += w l2), and each output moves its
 # sums from r to its own centre once (five operations).
 OPS_PER_PSF_TAP_SPLIT = 3
-OPS_PER_PSF_INPUT_SPLIT = 5
+OPS_PER_PSF_INPUT_SPLIT = 4
 OPS_PER_PSF_OUTPUT_SPLIT = 5
+
+
+# The one-kernel evaluator's line of an extended spaxel: Eqs. 1-8 with a
+# ten-term arctangent polynomial and the closed-form sums, a reciprocal square
+# root and a power of two.
+LINE_OPS_PER_EXT_SPAXEL = 45
+LINE_MUFU_PER_EXT_SPAXEL = 2
 
 
 def split_pass_ops_per_output(taps):
@@ -73,14 +80,6 @@ UNFOLDED_FP32_PER_DATA_VOXEL = 47.0
 # GB300 (dram__bytes_read.sum + dram__bytes_write.sum of the fused launch);
 # reported only for a run at that tuning and with that kernel build.
 FUSED_TRAFFIC_400 = {(12, 512, 0): 1433600.0, (12, 512, 1): 1318400.0}
-# DRAM bytes (read + write) of one launch of the split path's line stage
-# per step size (models per step -> bytes), from a one-pass ncu capture of
-# `bench.py --quick --steps 5 --warmup 2` on a GB300 with the current kernel
-# build (dram__bytes_read.sum + dram__bytes_write.sum, mean over launches);
-# 36 975 B read + 9 604 B written per launch of 80 models, the mean of 60
-# launches.
-SPLIT_LINE_TRAFFIC = {400: 46579.0}
-SPLIT_LINE_TRAFFIC_MODELS = 80  # models per line-stage launch of a 400-model step
 FLUSH_BYTES = 256 << 20
 
 
@@ -1233,9 +1232,8 @@ def run_gbk(args):
         stage_mean = np.mean(np.array(stage_reps), axis=0)
         out["gpu_launches"] = K * nl
         out["stages"] = [{"stage": name, "kernel": kern, "ms_per_step": float(t), "share": float(t / sum(stage_mean))}
-                         for name, kern, t in zip(("set-up", "line sums + PSF along x", "PSF along y + moments + chi2"),
-                                                  ("split_setup_kernel", "split_line_kernel", "split_psf_kernel"),
-                                                  stage_mean)]
+                         for name, kern, t in zip(("counters", "lines + PSF + moments + chi2"),
+                                                  ("memset", "tile_kernel"), stage_mean[:2])]
     if staged:
         out["config"]["path"] = "staged"
     if args.quick:
@@ -1279,13 +1277,14 @@ def run_gbk(args):
         return
 
     if split:
-        # ---- roofline of the dominant kernel: the line stage, ALU bound ----
-        # Algorithmic work per model: the line sampling (5 FP32 + 1 ex2 per
-        # extended voxel) and the PSF pass along x of every extended row
-        # (6 FP32 per tap per output, ey x nx outputs).
+        # ---- roofline of the evaluator's kernel: ALU bound ----
+        # Algorithmic work per model: the geometry and the closed-form line of
+        # every extended spaxel, the two PSF passes (ey x nx and ny x nx
+        # outputs) and the moments, residuals and chi2 of every data spaxel.
         taps = 2 * ((ex - g.nx) // 2) + 1
-        fma_a = FMA_OPS_PER_EXT_VOXEL * ex * ey * ez + split_pass_ops_per_output(taps) * ey * g.nx
-        mufu_a = MUFU_OPS_PER_EXT_VOXEL * ex * ey * ez
+        fma_a = (LINE_OPS_PER_EXT_SPAXEL * ex * ey + split_pass_ops_per_output(taps) * (ey + g.ny) * g.nx
+                 + OPS_PER_DATA_SPAXEL * g.nx * g.ny)
+        mufu_a = LINE_MUFU_PER_EXT_SPAXEL * ex * ey
         r32, r32x2, rmu = gbk.gbk_measure_alu_peak(stream)
         rfma = max(r32, r32x2)
         t_min = max(fma_a / rfma, mufu_a / rmu)
@@ -1294,28 +1293,16 @@ def run_gbk(args):
         achieved_ops = (fma_a + mufu_a) * n / t_a
         out["roofline"] = {
             "bound": "alu", "achieved": achieved_ops / 1e12, "peak": peak_ops / 1e12, "unit": "Tops/s",
-            "frac": achieved_ops / peak_ops, "traffic": SPLIT_LINE_TRAFFIC.get(n),
-            "traffic_note": ("DRAM bytes per launch (%d models) from one ncu capture of this kernel build: its "
-                             "x-filtered planes stay in L2" % SPLIT_LINE_TRAFFIC_MODELS if n in SPLIT_LINE_TRAFFIC
-                             else "no capture of this kernel build at this batch size"),
-            "kernel": "split_line_kernel",
-            "basis": "per model %.1f M FP32 + %.1f M ex2 lane ops: %d FP32 + %d ex2 per extended voxel (%d x %d x "
-                     "%d), %.1f FP32 per output of the PSF pass along x (%d taps x %d FMAs, %d per input and %d per "
-                     "output for the re-centring; %d x %d outputs); its time per step from CUDA events around each "
-                     "launch (%.3f ms of %.3f); measured FP32 pipe %.1f T lane-ops/s (scalar %.1f, f32x2 %.1f), "
-                     "ex2 %.1f T/s"
-                     % (fma_a / 1e6, mufu_a / 1e6, FMA_OPS_PER_EXT_VOXEL, MUFU_OPS_PER_EXT_VOXEL, ex, ey, ez,
+            "frac": achieved_ops / peak_ops, "traffic": None, "kernel": "tile_kernel",
+            "basis": "per model %.1f M FP32 + %.2f M MUFU lane ops: %d FP32 + %d MUFU per extended spaxel (%d x %d), "
+                     "%.1f FP32 per output of a PSF pass (%d taps x %d FMAs, %d per input and %d per output for the "
+                     "re-centring; %d x %d and %d x %d outputs), %d per data spaxel; measured FP32 pipe %.1f T "
+                     "lane-ops/s (scalar %.1f, f32x2 %.1f), ex2 %.1f T/s"
+                     % (fma_a / 1e6, mufu_a / 1e6, LINE_OPS_PER_EXT_SPAXEL, LINE_MUFU_PER_EXT_SPAXEL, ex, ey,
                         split_pass_ops_per_output(taps), taps, OPS_PER_PSF_TAP_SPLIT, OPS_PER_PSF_INPUT_SPLIT,
-                        OPS_PER_PSF_OUTPUT_SPLIT, ey, g.nx, t_a * 1e3,
-                        sum(st["ms_per_step"] for st in out["stages"]),
+                        OPS_PER_PSF_OUTPUT_SPLIT, ey, g.nx, g.ny, g.nx, OPS_PER_DATA_SPAXEL,
                         rfma / 1e12, r32 / 1e12, r32x2 / 1e12, rmu / 1e12),
             "peak_source": "measured on this device by gbk_measure_alu_peak"}
-        # the whole step on the same basis (both stages, every launch)
-        fma_all = fma_a + split_pass_ops_per_output(taps) * g.ny * g.nx + OPS_PER_DATA_SPAXEL * g.nx * g.ny
-        out["roofline_whole_step"] = {
-            "achieved": (fma_all + mufu_a) * n / (ms_step * 1e-3) / 1e12, "unit": "Tops/s",
-            "frac": (fma_all + mufu_a) * n / (ms_step * 1e-3) / ((fma_all + mufu_a) / max(fma_all / rfma, mufu_a / rmu)),
-            "basis": "both stages: %.1f M FP32 + %.1f M ex2 per model over the step time" % (fma_all / 1e6, mufu_a / 1e6)}
     if not split:
         # ---- roofline of the fused kernel: ALU (FP32 pipe + MUFU ex2) ----
         # Algorithmic work per model of the folded method: the line sampling

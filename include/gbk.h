@@ -132,11 +132,12 @@ typedef struct gbk_obs {
  *                   never leaves the SM; needs no workspace.
  *  GBK_PATH_STAGED  model cube -> separable convolution -> moments, each
  *                   stage through HBM (the paper's pipeline).
- *  GBK_PATH_SPLIT   two kernels: each extended spaxel's line folded into a
- *                   moment triplet (16 bytes, in the workspace, sized to stay
- *                   in L2), then the PSF passes, moments and chi-squared in
- *                   tiles; the cube is never formed.  Cube model, u = 1, PSF
- *                   radius <= 8 px.
+ *  GBK_PATH_SPLIT   one kernel, a CTA per model or tile of its image: each
+ *                   extended spaxel's line folded into a moment triplet in
+ *                   closed form, then the PSF passes, moments and chi-squared,
+ *                   all on chip; the cube is never formed.  Cube model, u = 1,
+ *                   PSF radius <= 8 px.  The workspace holds the chi-squared
+ *                   parts of tiled images.
  *  GBK_PATH_AUTO    the split path when it serves the geometry and the
  *                   workspace holds what it needs, else the fused path when
  *                   it serves the geometry, else the staged path. */
@@ -193,8 +194,7 @@ GBK_API gbk_status gbk_chi2(const gbk_geom *g, int32_t n_models, const double *p
 
 /* gbk_chi2 on the split path with every array in HOST memory (Eq. 11; the
  * call a user with data on the host makes): the parameters are copied on
- * `stream`, the observed maps on the split evaluator's second stream so that
- * their copy overlaps the first line stage (which does not read them), and
+ * `stream`, the observed maps beside them on a second stream, and
  * chi2 comes back on `stream`.  Asynchronous: host buffers must stay valid
  * until the stream has passed the call; pinned buffers make the copies
  * asynchronous, pageable ones are copied synchronously by the runtime.
@@ -233,14 +233,12 @@ GBK_API gbk_status gbk_chi2_host(const gbk_geom *g, int32_t n_models, const doub
 GBK_API gbk_status gbk_chi2_noalloc(const gbk_geom *g, int32_t n_models, const double *params,
                                     const gbk_obs *obs, double *chi2, float *resid, void *stream);
 
-/* gbk_chi2 on the split path (GBK_PATH_SPLIT), timed per stage with CUDA
- * events recorded on `stream` around every launch: stage_ms (host [3])
- * receives the milliseconds of the set-up kernel, of the line stage (the
- * Gaussian lines folded into moment triplets and the PSF along x,
- * Sec. 2.2.2-2.2.3) and of the PSF-along-y stage with the moments and chi2
- * (Sec. 2.2.3-2.2.6), each summed over the model chunks; launches (host, or
+/* gbk_chi2 on the split path (GBK_PATH_SPLIT), timed with CUDA events recorded
+ * on `stream`: stage_ms (host [3]) receives the milliseconds of clearing the
+ * arrival counters, of the evaluator (lines, PSF passes, moments and chi2,
+ * Sec. 2.2.2-2.2.6) and 0 (the path has no third stage); launches (host, or
  * NULL) the number of kernel launches.  Workspace as for gbk_chi2 on the split
- * path; at most 31 chunks; synchronises `stream`. */
+ * path; synchronises `stream`. */
 GBK_API gbk_status gbk_split_stage_times(const gbk_geom *g, int32_t n_models, const double *params,
                                          const gbk_obs *obs, double *chi2, void *workspace, size_t ws_bytes,
                                          float *stage_ms, int32_t *launches, void *stream);
@@ -638,9 +636,8 @@ GBK_API gbk_status gbk_measure_alu_peak(double *ffma_lane_ops_per_s, double *ffm
  * when a TMA load of the staged convolution did not complete in time, bit 1
  * when a pipeline wait of the tensor-core GEMM did not (the affected blocks
  * stopped early and their output is incomplete), bit 2 when the wait of
- * gbk_wait_selfcheck ran out, bit 3 when a tile load of the PSF stage of the
- * split path or of the split Jacobian did not complete in time (that model's
- * outputs are not written).
+ * gbk_wait_selfcheck ran out, bit 3 when a tile load of the split Jacobian's
+ * PSF stage did not complete in time (that model's outputs are not written).
  * Synchronising. */
 GBK_API gbk_status gbk_device_status(int32_t *status);
 

@@ -10,6 +10,7 @@
 #include "gbk_api_internal.h"
 #include "k_fused.h"
 #include "k_split.h"
+#include "k_tile.h"
 #include "k_tsplit.h"
 #include "k_gemm.h"
 #include "k_staged.h"
@@ -181,12 +182,12 @@ const char *gbk_version(void) { return "gbk 0.1 (sm_103a)"; }
 gbk_status gbk_device_status(int32_t *status)
 {
     if (!status) return fail(GBK_EINVAL, "status is NULL");
-    int c = 0, c2 = 0, g = 0, w = 0, sp = 0, ts = 0;
+    int c = 0, c2 = 0, g = 0, w = 0, ts = 0;
     gbk_status s;
     if ((s = conv_status_read(&c)) || (s = conv_fir_status_read(&c2)) || (s = gemm_status_read(&g)) ||
-        (s = selfcheck_status_read(&w)) || (s = split_status_read(&sp)) || (s = tsplit_status_read(&ts)))
+        (s = selfcheck_status_read(&w)) || (s = tsplit_status_read(&ts)))
         return s;
-    *status = ((c || c2) ? 1 : 0) | (g ? 2 : 0) | (w ? 4 : 0) | ((sp || ts) ? 8 : 0);
+    *status = ((c || c2) ? 1 : 0) | (g ? 2 : 0) | (w ? 4 : 0) | (ts ? 8 : 0);
     return ok();
 }
 
@@ -276,7 +277,18 @@ static gbk_status run_fused(const Geom &g, int32_t n, const double *params, floa
     a.chi2 = chi2;
     a.resid = resid;
     if (n == 0) return ok();
-    gbk_status s = launch_fused(a, st);
+    // The one-kernel evaluator where it needs no workspace either: without
+    // chi2 any image, with it an image that fits one CTA (its chi2 parts have
+    // nowhere to meet).  A call for the maps of 77 models of 57 x 43 x 37,
+    // alone: 58 us on the cluster kernel, 43 us on this one.  A geometry whose
+    // cluster launch was tuned keeps it.
+    TileShape ts;
+    gbk_status s;
+    if (g.ex <= 1024 && !fused_tuned(g) && tile_shape(g, chi2 ? kTileChi2Batch : n, chi2 != nullptr, &ts) &&
+        n <= 0x7fffffff / ts.tiles)
+        s = launch_tile(g, ts, n, params, obs, maps, chi2, resid, TileScratch(), nullptr, 0, st);
+    else
+        s = launch_fused(a, st);
     if (s) return s;
     return ok();
 }
@@ -387,10 +399,9 @@ gbk_status gbk_chi2_host(const gbk_geom *gin, int32_t n_models, const double *pa
     float *d_maps = (float *)(ws + L.maps);
     uint8_t *d_mask = (uint8_t *)(ws + L.mask);
     const gbk_obs d_obs = {d_maps, d_maps + np, d_maps + 2 * np, d_maps + 3 * np, d_mask};
-    // The parameters go on the caller's stream (the line stage needs them);
-    // the maps on the PSF stages' stream, after everything the caller's
-    // stream holds (an earlier call's PSF stage may still read this
-    // workspace), so that their copy overlaps the line stage.
+    // The parameters go on the caller's stream, the maps beside them on the
+    // auxiliary stream, after everything the caller's stream holds (an
+    // earlier call's evaluator may still read this workspace).
     cudaError_t e;
     if ((e = cudaMemcpyAsync(d_params, params, sizeof(double) * GBK_NPAR * n_models, cudaMemcpyDefault, st)) ||
         (e = cudaEventRecord(aux->start, st)) || (e = cudaStreamWaitEvent(aux->s, aux->start, 0)) ||
@@ -404,8 +415,8 @@ gbk_status gbk_chi2_host(const gbk_geom *gin, int32_t n_models, const double *pa
     if ((s = launch_split(g, n_models, d_params, &d_obs, nullptr, d_chi2, nullptr, ws + L.split, L.total - L.split, st,
                           nullptr, nullptr, aux->obs)))
         return s;
-    // the last PSF stage is joined to st (or ran on it after the maps'
-    // event), so the maps' stream holds nothing past this point
+    // the evaluator ran on st after the maps' event, so the maps' stream
+    // holds nothing past this point
     if ((e = cudaMemcpyAsync(chi2, d_chi2, sizeof(double) * n_models, cudaMemcpyDefault, st)))
         return cuda_fail(e, "gbk_chi2_host: chi2 to the host");
     return ok();

@@ -57,6 +57,8 @@ struct FusedConfig {
 size_t fused_smem_bytes_host(const Geom &g, int band);
 bool fused_config_ragged(const Geom *geoms, int n, int cs, int threads, size_t *smem);
 bool fused_config(const Geom &g, FusedConfig *cfg);
+// A tuning was set for this geometry (by the caller or the autotuner).
+bool fused_tuned(const Geom &g);
 bool fused_config_valid(const Geom &g, int cs, int threads, int persistent, FusedConfig *cfg);
 gbk_status launch_fused(const FusedArgs &args, cudaStream_t stream);
 // Velocity-field models (k_vfield.cu); launch_fused dispatches to it.

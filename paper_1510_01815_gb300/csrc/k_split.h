@@ -1,4 +1,4 @@
-// k_split.h -- launcher of the two-stage fused evaluator (k_split.cu).
+// k_split.h -- the split path's workspace and launcher (k_split.cu).
 #pragma once
 
 #include <cuda.h>
@@ -7,22 +7,21 @@
 
 namespace gbk {
 
-constexpr int kSplitMaxR = 8;  // largest PSF radius the PSF stage is compiled for
+constexpr int kSplitMaxR = 8;  // largest PSF radius served
 
-// Geometries the two-stage evaluator serves (cube model, u = 1, R <= 8).
+// Geometries the split path serves (cube model, u = 1, R <= 8).
 bool split_supported(const Geom &g);
 // Workspace of a call over n_models (0 when the geometry is not served).
 size_t split_workspace_bytes(const Geom &g, int n_models);
 // chi2 (and optionally maps and residuals) of n models; asynchronous on st.
-// CUDA events recorded on the launch stream around every launch of a call
-// (start, after the set-up, after each stage-A and stage-B launch), for the
-// per-stage timings of gbk_split_stage_times.
+// CUDA events recorded on the launch stream (start, after the clearing of the
+// counters, end), for gbk_split_stage_times.
 struct SplitTimer {
-    cudaEvent_t ev[64] = {};
-    int n = 0;
+    cudaEvent_t ev[4] = {};
+    int n = 0, launches = 0;
     cudaError_t mark(cudaStream_t st)
     {
-        if (n >= 64) return cudaErrorInvalidValue;
+        if (n >= 4) return cudaErrorInvalidValue;
         cudaError_t e = cudaEventCreate(&ev[n]);
         if (e != cudaSuccess) return e;
         return cudaEventRecord(ev[n++], st);
@@ -51,9 +50,6 @@ struct SplitAux {
 };
 gbk_status split_aux(SplitAux **out);
 
-// Reads and clears the PSF stage's TMA wait status (1 = a load timed out).
-gbk_status split_status_read(int *v);
-
 // A batched call's galaxies: models i*mpg .. i*mpg + mpg - 1 belong to galaxy
 // i, which is compared with obs_list[i] (device, or null: *obs for all) and
 // left alone when skip[i] != 0 (device, or null).
@@ -62,8 +58,8 @@ struct SplitBatch {
     const int32_t *skip;
     int mpg;
 };
-// obs_ready (or null): an event the first PSF stage waits for (the observed
-// maps' copy); the line stages do not read the maps.
+// obs_ready (or null): an event the evaluator waits for (the observed maps'
+// copy).
 gbk_status launch_split(const Geom &g, int n, const double *params, const gbk_obs *obs, float *maps, double *chi2,
                         float *resid, void *ws, size_t ws_bytes, cudaStream_t st, SplitTimer *timer = nullptr,
                         const SplitBatch *batch = nullptr, cudaEvent_t obs_ready = nullptr);

@@ -2,7 +2,10 @@
 // channel width and LSF in one batch), the setting of the survey-scale
 // fitting Bekiaris et al. 2015 motivate in Sec. 1 and Sec. 5.
 //
-// Two ways to serve a survey with the fused evaluator:
+// A galaxy whose image fits one CTA goes to the one-kernel evaluator
+// (k_tile.cu): one launch per PSF radius and CTA size, costliest galaxy
+// first from a work counter.  The others, and surveys with a tuning, take the
+// cluster evaluator (k_fused.cu) in one of two ways:
 //  * one persistent launch: a resident wave of thread-block clusters of one
 //    size (the smallest that fits every galaxy two CTAs to an SM) takes the
 //    models, costliest galaxy first, from a work counter as each cluster
@@ -23,6 +26,7 @@
 #include "gbk_api_internal.h"
 #include "k_fused.h"
 #include "k_tangent.h"
+#include "k_tile.h"
 #include "k_tsplit.h"
 #include "survey.h"
 
@@ -32,6 +36,10 @@ static size_t al256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 // Shared memory per CTA that lets two CTAs of 512 threads share an SM.
 constexpr size_t kSurveySmemCap = 228 * 1024 / 2 - 3 * 1024;
+
+// Work counters at the end of the tables: a persistent cluster launch's two,
+// then one for each tile class (at most five CTA sizes and nine PSF radii).
+constexpr int kSurveyCounters = 64;
 
 // One persistent launch unless a survey tuning says otherwise.
 constexpr int kSurveyDefaultOne = 1;
@@ -91,6 +99,76 @@ static int one_launch_cs(const std::vector<Geom> &geo, int threads, size_t *smem
     return 0;
 }
 
+// One cluster launch per group of galaxies order[beg .. end) of the same
+// cluster and block size.
+static gbk_status cluster_groups(SurveyPlan *sp, int beg, int end, const std::vector<int> &cs_of,
+                                 const std::vector<int> &thr_of)
+{
+    for (int k = beg; k < end;) {
+        int i0 = sp->order[k], e = k;
+        while (e < end && cs_of[sp->order[e]] == cs_of[i0] && thr_of[sp->order[e]] == thr_of[i0]) ++e;
+        SurveyClass c;
+        c.cs = cs_of[i0];
+        c.threads = thr_of[i0];
+        c.beg = k;
+        c.end = e;
+        c.persistent = 0;
+        c.n_solo = 0;
+        std::vector<Geom> members;
+        for (int j = k; j < e; ++j) members.push_back(sp->geo[sp->order[j]]);
+        if (!fused_config_ragged(members.data(), (int)members.size(), c.cs, c.threads, &c.smem))
+            return fail(GBK_EUNSUPPORTED, "survey class with %d-CTA clusters does not fit", c.cs);
+        sp->classes.push_back(c);
+        k = e;
+    }
+    return GBK_OK;
+}
+
+// Moves the galaxies that the one-kernel evaluator serves to classes of their
+// own, by CTA size (largest first: the launches run one after the other, and
+// the last one's tail is the short items') and PSF radius; the others stay on
+// the cluster evaluator.  A survey of 2048 galaxies of 24 - 96 spaxels took
+// 546 us on one cluster launch, 243 us on these.
+template <class Cost>
+static gbk_status tile_classes(SurveyPlan *sp, const std::vector<int> &cs_of, const std::vector<int> &thr_of,
+                               const Cost &cost)
+{
+    const int n = sp->n_gal;
+    std::vector<int> thr(n);
+    std::vector<size_t> smem(n);
+    int served = 0;
+    for (int i = 0; i < n; ++i) served += (thr[i] = tile_ragged_threads(sp->geo[i], &smem[i])) > 0;
+    if (!served) return GBK_OK;
+    std::stable_sort(sp->order.begin(), sp->order.end(), [&](int a, int b) {
+        if ((thr[a] > 0) != (thr[b] > 0)) return thr[a] == 0;
+        if (thr[a] == 0) {
+            if (cs_of[a] != cs_of[b]) return cs_of[a] > cs_of[b];
+            if (thr_of[a] != thr_of[b]) return thr_of[a] > thr_of[b];
+        } else {
+            if (thr[a] != thr[b]) return thr[a] > thr[b];
+            if (sp->geo[a].R != sp->geo[b].R) return sp->geo[a].R > sp->geo[b].R;
+        }
+        if (cost(a) != cost(b)) return cost(a) > cost(b);
+        return a < b;
+    });
+    sp->classes.clear();
+    gbk_status s = cluster_groups(sp, 0, n - served, cs_of, thr_of);
+    if (s) return s;
+    for (int k = n - served; k < n;) {
+        const int i0 = sp->order[k];
+        SurveyClass c = {};
+        c.tile = 1;
+        c.R = sp->geo[i0].R;
+        c.threads = thr[i0];
+        c.beg = k;
+        for (; k < n && thr[sp->order[k]] == c.threads && sp->geo[sp->order[k]].R == c.R; ++k)
+            c.smem = std::max(c.smem, smem[sp->order[k]]);
+        c.end = k;
+        sp->classes.push_back(c);
+    }
+    return GBK_OK;
+}
+
 gbk_status survey_plan(const gbk_geom *geoms, int n_gal, SurveyPlan *sp, const SurveyTuning *force)
 {
     if (!geoms) return fail(GBK_EINVAL, "geoms is NULL");
@@ -126,12 +204,16 @@ gbk_status survey_plan(const gbk_geom *geoms, int n_gal, SurveyPlan *sp, const S
     }
     auto cost = [&](int i) { const Geom &g = sp->geo[i]; return (long long)g.ex * g.ey * g.ez; };
     SurveyTuning tu = {kSurveyDefaultOne, 0, 512};
+    bool tuned = force != nullptr;
     if (force) {
         tu = *force;
     } else if (n_gal > 0) {
         std::lock_guard<std::mutex> lk(g_stune_mu);
         auto it = g_stune.find(survey_key(sp->geo));
-        if (it != g_stune.end()) tu = it->second;
+        if (it != g_stune.end()) {
+            tu = it->second;
+            tuned = true;
+        }
     }
     sp->order.resize(n_gal);
     std::iota(sp->order.begin(), sp->order.end(), 0);
@@ -192,22 +274,13 @@ gbk_status survey_plan(const gbk_geom *geoms, int n_gal, SurveyPlan *sp, const S
             return cost(a) > cost(b);
         });
     sp->tuning = tu;
-    for (int k = 0; k < n_gal && !tu.one;) {
-        int i0 = sp->order[k], e = k;
-        while (e < n_gal && cs_of[sp->order[e]] == cs_of[i0] && thr_of[sp->order[e]] == thr_of[i0]) ++e;
-        SurveyClass c;
-        c.cs = cs_of[i0];
-        c.threads = thr_of[i0];
-        c.beg = k;
-        c.end = e;
-        c.persistent = 0;
-        c.n_solo = 0;
-        std::vector<Geom> members;
-        for (int j = k; j < e; ++j) members.push_back(sp->geo[sp->order[j]]);
-        if (!fused_config_ragged(members.data(), (int)members.size(), c.cs, c.threads, &c.smem))
-            return fail(GBK_EUNSUPPORTED, "survey class with %d-CTA clusters does not fit", c.cs);
-        sp->classes.push_back(c);
-        k = e;
+    if (!tu.one) {
+        gbk_status s = cluster_groups(sp, 0, n_gal, cs_of, thr_of);
+        if (s) return s;
+    }
+    if (!tuned) {
+        gbk_status s = tile_classes(sp, cs_of, thr_of, cost);
+        if (s) return s;
     }
     // classes of the analytic Jacobian kernel: smallest cluster whose CTAs fit
     std::vector<int> tcs(n_gal);
@@ -247,7 +320,7 @@ gbk_status survey_plan(const gbk_geom *geoms, int n_gal, SurveyPlan *sp, const S
     }
     sp->table_bytes = n_gal == 0 ? 0
                                  : al256(sizeof(Geom) * n_gal) + al256(sizeof(int64_t) * (n_gal + 1)) +
-                                       2 * al256(sizeof(int32_t) * n_gal) + al256(2 * sizeof(int));
+                                       2 * al256(sizeof(int32_t) * n_gal) + al256(kSurveyCounters * sizeof(int));
     return GBK_OK;
 }
 
@@ -382,8 +455,24 @@ gbk_status survey_eval(const SurveyPlan &sp, int mpg, const double *params, cons
 {
     const std::vector<SurveyClass> &classes = live ? live->classes : sp.classes;
     const int32_t *d_order = live ? live->d_order : sp.d_order;
+    // counters: 0 and 1 for a persistent cluster launch, then one per tile class
+    int tiles = 0;
+    for (const SurveyClass &c : classes) tiles += c.tile;
+    if (tiles > kSurveyCounters - 2) return fail(GBK_EUNSUPPORTED, "survey: %d launch classes", tiles);
+    if (tiles) {
+        cudaError_t e = cudaMemsetAsync(sp.d_work + 2, 0, tiles * sizeof(int), st);
+        if (e != cudaSuccess) return cuda_fail(e, "survey: resetting the work counters");
+    }
+    int *work = sp.d_work + 2;
     for (size_t ci = 0; ci < classes.size(); ++ci) {
         const SurveyClass &c = classes[ci];
+        if (c.tile) {
+            const TileRagged t = {sp.d_geo, sp.d_pix_off, d_order + c.beg, params, obs_list, skip, maps, chi2, resid,
+                                  work++,   (c.end - c.beg) * mpg,          mpg};
+            gbk_status s = launch_tile_ragged(t, c.R, c.threads, c.smem, st);
+            if (s) return s;
+            continue;
+        }
         FusedArgs a = {};
         a.g = sp.geo[live ? live->rep[ci] : sp.order[c.beg]];
         a.n_models = (c.end - c.beg) * mpg;

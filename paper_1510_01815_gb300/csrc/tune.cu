@@ -90,6 +90,12 @@ static bool heuristic(const Geom &g, FusedConfig *cfg)
     return best > 0.0;
 }
 
+bool fused_tuned(const Geom &g)
+{
+    std::lock_guard<std::mutex> lk(g_tune_mu);
+    return g_tune_cache.find(key_of(g)) != g_tune_cache.end();
+}
+
 bool fused_config(const Geom &g, FusedConfig *cfg)
 {
     if (g.u != 1) return false;
