@@ -57,7 +57,16 @@ struct CnnTables {
     size_t off[kCnnL + 1];
     __nv_bfloat16 *W[kCnnL], *WT[kCnnL];
     float *bias[kCnnL];
+    __nv_bfloat16 *W0q;  // the first layer's weights four times, block-diagonal [4 C_0][4 K_0]
+    float *bias0q;       // and its biases four times
 };
+
+// The first layer runs on four rows at a time: its patch matrix [M][16] read
+// as [M / 4][64] against four copies of the weights on the diagonal is the
+// same product (the added terms are exact zeros) with full 128-byte rows for
+// the tensor copies; as 32-byte rows of a 64-wide box, most of it fill, they
+// set the time (1048576 x 32 x 16 with one epilogue: 102 us, so 78 us).
+constexpr int kCnnQ = 4;
 
 __device__ __forceinline__ uint64_t sm_mix(uint64_t z)
 {
@@ -109,30 +118,47 @@ __global__ void cnn_init_kernel(float *P, CnnTables t, uint64_t seed)
     }
 }
 
-// BF16 copies of the weights (row-major and transposed) and FP32 biases.
-__global__ void cnn_publish_kernel(const float *P, CnnTables t)
+// BF16 copies of the weights (row-major, and transposed for a backward pass)
+// and FP32 biases; for a backward pass also the rows of ones under the
+// transposed activations (ones[l], M[l] values, l >= 1).
+struct CnnOnes {
+    __nv_bfloat16 *row[kCnnL];
+    unsigned n[kCnnL];
+};
+
+__global__ void cnn_publish_kernel(const float *P, CnnTables t, bool backward, CnnOnes ones)
 {
-    const size_t n = t.off[kCnnL];
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+    const unsigned n = (unsigned)t.off[kCnnL], first = blockIdx.x * blockDim.x + threadIdx.x,
+                   step = gridDim.x * blockDim.x;
+    for (unsigned i = first; i < n; i += step) {
         int l = 0;
-        while (i >= t.off[l + 1]) ++l;
-        const size_t j = i - t.off[l];
-        const int K = t.K[l], C = t.C[l];
-        const int o = (int)(j / (size_t)(K + 1)), k = (int)(j % (size_t)(K + 1));
+        while (i >= (unsigned)t.off[l + 1]) ++l;
+        const unsigned j = i - (unsigned)t.off[l];
+        const unsigned K = t.K[l], C = t.C[l];
+        const unsigned o = j / (K + 1), k = j - o * (K + 1);
         const float v = P[i];
         if (k == K) {
             t.bias[l][o] = v;
+            if (l == 0)
+                for (unsigned q = 0; q < kCnnQ; ++q) t.bias0q[q * C + o] = v;
         } else {
             const __nv_bfloat16 h = __float2bfloat16_rn(v);
             t.W[l][(size_t)o * K + k] = h;
-            t.WT[l][(size_t)k * C + o] = h;
+            if (l == 0)
+                for (unsigned q = 0; q < kCnnQ; ++q)
+                    for (unsigned p = 0; p < kCnnQ; ++p)
+                        t.W0q[(size_t)(q * C + o) * (kCnnQ * K) + p * K + k] = p == q ? h : __float2bfloat16_rn(0.f);
+            if (backward) t.WT[l][(size_t)k * C + o] = h;
         }
     }
+    if (!backward) return;
+    for (int l = 1; l < kCnnL; ++l)
+        for (unsigned i = first; i < ones.n[l]; i += step) ones.row[l][i] = __float2bfloat16_rn(1.f);
 }
 
 // Input encoding: sample b, 2 x 2 patch (Y, X) -> row b * 1024 + morton(Y, X);
-// column (dy * 2 + dx) * 4 + ch.  Also the transposed matrix with a row of
-// ones at index 16.  One thread per patch: two 8-byte loads each of v and
+// column (dy * 2 + dx) * 4 + ch.  With AT also the transposed matrix with a row
+// of ones at index 16.  One thread per patch: two 8-byte loads each of v and
 // sigma and two 2-byte mask loads, one 32-byte row store, and 17 transposed
 // stores that are coalesced across the warp (consecutive threads, consecutive
 // rows).
@@ -171,32 +197,30 @@ __global__ void cnn_encode_kernel(int n, const float *v, const float *s, const u
         const uint4 *src = reinterpret_cast<const uint4 *>(h);
         dst[0] = src[0];
         dst[1] = src[1];
+        if (!AT) continue;
 #pragma unroll
         for (int e = 0; e < kK; ++e) AT[(size_t)e * rows + r] = h[e];
         AT[(size_t)kK * rows + r] = __float2bfloat16_rn(1.f);
     }
 }
 
-__global__ void cnn_ones_kernel(__nv_bfloat16 *row, size_t n)
-{
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        row[i] = __float2bfloat16_rn(1.f);
-}
-
 // Loss = mean over samples and the 10 used outputs of (y - t)^2; dY = dL/dy
-// (BF16, plain and transposed).  One block; fixed-order reduction.
-__global__ void cnn_loss_kernel(const float *Y, const float *T, int B, __nv_bfloat16 *dY, __nv_bfloat16 *dYT,
-                                float *loss)
+// (BF16, plain and transposed).  Each block leaves its part of the loss (FP64:
+// on one SM the squares alone took 8 us) for cnn_loss_sum_kernel, which adds
+// them in order.
+__global__ void __launch_bounds__(256) cnn_loss_kernel(const float *Y, const float *T, int B, __nv_bfloat16 *dY,
+                                                       __nv_bfloat16 *dYT, double *part)
 {
-    __shared__ double red[32];
+    __shared__ double red[8];
     double acc = 0.0;
     const float g = 2.f / (float)(B * kCnnTargets);
-    for (int i = threadIdx.x; i < B * kCnnOut; i += blockDim.x) {
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i < B * kCnnOut) {
         const int b = i / kCnnOut, j = i % kCnnOut;
         float d = 0.f;
         if (j < kCnnTargets) {
             d = Y[(size_t)b * kCnnOut + j] - T[(size_t)b * kCnnTargets + j];
-            acc += (double)d * d;
+            acc = (double)d * d;
         }
         const __nv_bfloat16 h = __float2bfloat16_rn(g * d);
         dY[(size_t)b * kCnnOut + j] = h;
@@ -207,9 +231,17 @@ __global__ void cnn_loss_kernel(const float *Y, const float *T, int B, __nv_bflo
     __syncthreads();
     if (threadIdx.x == 0) {
         double s = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-        if (loss) *loss = (float)(s / (double)(B * kCnnTargets));
+        for (int w = 0; w < 8; ++w) s += red[w];
+        part[blockIdx.x] = s;
     }
+}
+
+__global__ void cnn_loss_sum_kernel(const double *part, int n, int B, float *loss)
+{
+    double s = 0.0;
+    for (int i = threadIdx.x; i < n; i += 32) s += part[i];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) *loss = (float)(s / (double)(B * kCnnTargets));
 }
 
 __global__ void cnn_adam_kernel(float *P, float *Mo, float *Vo, const float *G, size_t n, float lr, float b1, float b2,
@@ -304,6 +336,11 @@ struct CnnWs {
     size_t total;
 };
 
+// Row length of a weight gradient's split-K slices: K + 1 padded so that the
+// rows take 16-byte stores (scalar ones, a row per lane, wrote 4 of every 32
+// bytes they touched).
+static int slice_ld(int l) { return (kCnnK[l] + 1 + 3) & ~3; }
+
 static int split_of(int l, int B, int *kt_split)
 {
     const int M = kCnnC[l], N = kCnnK[l] + 1, Kc = B * kCnnRows[l];
@@ -339,7 +376,7 @@ static CnnWs cnn_layout(int B, char *base)
     for (int l = 0; l < kCnnL; ++l) {
         int kts;
         const int sp = split_of(l, B, &kts);
-        const size_t need = (size_t)sp * kCnnC[l] * (kCnnK[l] + 1);
+        const size_t need = (size_t)sp * kCnnC[l] * slice_ld(l);
         if (need > w.part_floats) w.part_floats = need;
     }
     w.part = (float *)take(sizeof(float) * w.part_floats);
@@ -353,6 +390,8 @@ static CnnWs cnn_layout(int B, char *base)
         w.t.bias[l] = (float *)take(sizeof(float) * kCnnC[l]);
     }
     w.t.off[kCnnL] = param_count();
+    w.t.W0q = (__nv_bfloat16 *)take(bf * kCnnQ * kCnnC[0] * kCnnQ * kCnnK[0]);
+    w.t.bias0q = (float *)take(sizeof(float) * kCnnQ * kCnnC[0]);
     w.total = o;
     return w;
 }
@@ -398,15 +437,28 @@ static gbk_status cnn_forward_ws(const CnnWs &w, int B, bool want_transposed, cu
             a.out_f32 = w.Y;
             a.ldo = kCnnOut;
         }
-        if ((s = gemm(w.A[l], kCnnK[l], w.t.W[l], kCnnK[l], a, st))) return s;
+        const __nv_bfloat16 *W = w.t.W[l];
+        if (l == 0) {
+            // rows in fours (B kCnnRows[0] is a multiple of 4): the row-major
+            // output is the same memory, the transposed one a plain transpose
+            a.M /= kCnnQ;
+            a.N *= kCnnQ;
+            a.K *= kCnnQ;
+            a.ldo *= kCnnQ;
+            a.bias = w.t.bias0q;
+            a.t_log2 = 0;
+            W = w.t.W0q;
+        }
+        if ((s = gemm(w.A[l], a.K, W, a.K, a, st))) return s;
     }
     return GBK_OK;
 }
 
 static gbk_status cnn_encode(const CnnWs &w, int B, const float *v, const float *sg, const uint8_t *mask,
-                             cudaStream_t st)
+                             bool want_transposed, cudaStream_t st)
 {
-    cnn_encode_kernel<<<grid_for((size_t)B * kCnnRows[0]), 256, 0, st>>>(B, v, sg, mask, w.A[0], w.AT[0]);
+    cnn_encode_kernel<<<grid_for((size_t)B * kCnnRows[0]), 256, 0, st>>>(B, v, sg, mask, w.A[0],
+                                                                           want_transposed ? w.AT[0] : nullptr);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "CNN encode launch");
     return GBK_OK;
@@ -418,14 +470,19 @@ static gbk_status cnn_grad_ws(const CnnWs &w, const float *P, int B, const float
 {
     gbk_status s;
     const size_t np = param_count();
-    cnn_publish_kernel<<<grid_for(np), 256, 0, st>>>(P, w.t);
+    CnnOnes ones = {};
     for (int l = 1; l < kCnnL; ++l) {
         const size_t M = (size_t)B * kCnnRows[l];
-        cnn_ones_kernel<<<grid_for(M), 256, 0, st>>>(w.AT[l] + (size_t)kCnnK[l] * M, M);
+        ones.row[l] = w.AT[l] + (size_t)kCnnK[l] * M;
+        ones.n[l] = (unsigned)M;
     }
-    if ((s = cnn_encode(w, B, v, sg, mask, st))) return s;
+    cnn_publish_kernel<<<grid_for(np), 256, 0, st>>>(P, w.t, true, ones);
+    if ((s = cnn_encode(w, B, v, sg, mask, true, st))) return s;
     if ((s = cnn_forward_ws(w, B, true, st))) return s;
-    cnn_loss_kernel<<<1, 1024, 0, st>>>(w.Y, T, B, w.dY, w.dYT, w.loss);
+    // the parts lie in the split-K slices, which the backward pass fills later
+    const int lblocks = (B * kCnnOut + 255) / 256;
+    cnn_loss_kernel<<<lblocks, 256, 0, st>>>(w.Y, T, B, w.dY, w.dYT, (double *)w.part);
+    cnn_loss_sum_kernel<<<1, 32, 0, st>>>((const double *)w.part, lblocks, B, w.loss);
     for (int l = kCnnL - 1; l >= 0; --l) {
         const int M = B * kCnnRows[l], C = kCnnC[l], K = kCnnK[l];
         const __nv_bfloat16 *dZ = (l == kCnnL - 1) ? w.dY : w.dZ[l];
@@ -437,13 +494,13 @@ static gbk_status cnn_grad_ws(const CnnWs &w, const float *P, int B, const float
         g.K = M;
         g.alpha = 1.f;
         g.out_f32 = w.part;
-        g.ldo = K + 1;
+        g.ldo = slice_ld(l);
         int kts;
         const int splits = split_of(l, B, &kts);
         g.kt_split = kts;
-        g.split_stride = (size_t)C * (K + 1);
+        g.split_stride = (size_t)C * g.ldo;
         if ((s = gemm(dZT, M, w.AT[l], M, g, st))) return s;
-        if ((s = launch_splitk_reduce(w.part, splits, g.split_stride, C, K + 1, K + 1, w.G + param_offset(l), st)))
+        if ((s = launch_splitk_reduce(w.part, splits, g.split_stride, C, K + 1, g.ldo, K + 1, w.G + param_offset(l), st)))
             return s;
         if (l == 0) break;
         // dZ_{l-1} = (dZ_l W_l) * [A_l > 0], in A_l's layout, plus its transpose
@@ -572,8 +629,8 @@ gbk_status gbk_cnn_forward(const float *params, int32_t n, const float *v, const
     if ((s = check_device_ptr(workspace, "workspace", 256))) return s;
     w = cnn_layout(n, (char *)workspace);
     cudaStream_t st = (cudaStream_t)stream;
-    cnn_publish_kernel<<<grid_for(param_count()), 256, 0, st>>>(params, w.t);
-    if ((s = cnn_encode(w, n, v, sigma, mask, st))) return s;
+    cnn_publish_kernel<<<grid_for(param_count()), 256, 0, st>>>(params, w.t, false, CnnOnes());
+    if ((s = cnn_encode(w, n, v, sigma, mask, false, st))) return s;
     if ((s = cnn_forward_ws(w, n, false, st))) return s;
     cudaError_t e = cudaMemcpyAsync(out, w.Y, sizeof(float) * n * kCnnOut, cudaMemcpyDeviceToDevice, st);
     if (e != cudaSuccess) return cuda_fail(e, "CNN output copy");

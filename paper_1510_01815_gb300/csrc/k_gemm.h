@@ -11,7 +11,7 @@ namespace gbk {
 // A [M][lda], B [N][ldb] BF16 row-major; D BF16 and/or FP32 [M][ldo].
 struct GemmArgs {
     int M, N, K;
-    int bn;                       // output tile width (set by the launcher)
+    int bn, stages;               // output tile width, slabs in the ring (set by the launcher)
     float alpha;
     const float *bias;            // [N] or null
     int relu;
@@ -34,8 +34,9 @@ struct GemmArgs {
 
 gbk_status launch_gemm_bf16(const void *A, int lda, const void *B, int ldb, const GemmArgs &args, cudaStream_t st);
 gbk_status gemm_status_read(int *v);
-// Fixed-order sum of split-K slices: out[m][n] = sum_z part[z][m][n] (FP32, ld ldo).
-gbk_status launch_splitk_reduce(const float *part, int splits, size_t stride, int M, int N, int ldo, float *out,
+// Fixed-order sum of split-K slices: out[m][n] = sum_z part[z][m][n] (FP32,
+// leading dimensions ldp and ldo).
+gbk_status launch_splitk_reduce(const float *part, int splits, size_t stride, int M, int N, int ldp, int ldo, float *out,
                                 cudaStream_t st);
 
 }  // namespace gbk
