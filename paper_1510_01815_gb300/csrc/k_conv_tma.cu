@@ -8,12 +8,19 @@
 //     two channels ahead, into a double buffer, so the cube is read from HBM
 //     exactly once and the load overlaps the arithmetic;
 //   - the x pass gives each thread four adjacent outputs from one float4-
-//     loaded row segment; the y pass gives each thread four outputs of one
-//     column;
+//     loaded row segment (four taps per load); the y pass gives each thread
+//     2 x 2 outputs, two columns per packed f32x2 operation;
 //   - the z pass keeps, per owned spaxel, the 2 Rz + 1 partial output
 //     channels the current input channel contributes to in registers (a
 //     shifting window, template-sized), and writes a channel as soon as its
 //     window is complete -- coalesced rows of 32 floats.
+// Where the tiles alone do not fill the chip the channels are cut as well: a
+// CTA walks the extended channels of a range of output channels (the 2 Rz at
+// its ends are then read twice).  32 models of 64 x 64 x 128 fine voxels (R =
+// 9, Rz = 6) are 128 tiles: 206 us with one CTA each and scalar passes, 160 us
+// in halves, 124 us in halves with the passes as above (the whole call: 272 us
+// before, 190 us now).  Issue slots bound it: the x pass is scalar, since its
+// row pairs would start at odd columns for every other tap.
 // Waits on the mbarriers are bounded: a CTA that gives up records a status in
 // g_conv_status and stops (the host reports it as GBK_ECUDA via
 // gbk_device_status()).
@@ -37,8 +44,10 @@ struct ConvTmaArgs {
     int n_models;
     int tiles_x, tiles_y;
     int box_w;                     // TMA box width, >= 32 + 2R, multiple of 4
+    int zparts, zlen;              // ranges of output channels per tile, channels per range
     float *fine;                   // [n][nzf][nyf][nxf]
     size_t f_model_stride;
+    int vec2;                      // 1: output rows take 8-byte stores
 };
 
 template <int W>
@@ -49,8 +58,12 @@ __global__ void __launch_bounds__(kCThreads, (W <= 15 ? 2 : 1)) conv3d_tma_kerne
     const int R = g.R, Rz = g.Rz;
     const int SY = kCT + 2 * R, BW = a.box_w;
     const int tiles = a.tiles_x * a.tiles_y;
-    const int model = blockIdx.x / tiles;
-    const int t = blockIdx.x - model * tiles;
+    const int zpart = blockIdx.x % a.zparts, mt = blockIdx.x / a.zparts;
+    const int model = mt / tiles;
+    const int t = mt - model * tiles;
+    // output channels [k0, k1) come from extended channels [k0, k1 + 2 Rz)
+    const int k0 = zpart * a.zlen, k1 = min(g.nzf, k0 + a.zlen);
+    const int ne = k1 + 2 * Rz - k0;
     const int ty0 = (t / a.tiles_x) * kCT, tx0 = (t % a.tiles_x) * kCT;
     const int tid = threadIdx.x;
 
@@ -63,7 +76,9 @@ __global__ void __launch_bounds__(kCThreads, (W <= 15 ? 2 : 1)) conv3d_tma_kerne
     float *slab0 = csm;                        // [SY][BW]
     float *slab1 = slab0 + SS;
     float *X = slab1 + SS;                     // [SY][32] after the x pass
+    const int taps = (2 * R + 1 + 3) & ~3;
     float *wxy = X + SY * kCT;                 // 2R+1 taps (padded)
+    float *wdup = wxy + taps;                  // the same, each tap twice
     __shared__ __align__(8) uint64_t bar[2];
     __shared__ float s_wz[W];
     __shared__ int s_abort;
@@ -75,10 +90,15 @@ __global__ void __launch_bounds__(kCThreads, (W <= 15 ? 2 : 1)) conv3d_tma_kerne
         s_abort = 0;
     }
     // taps (each thread that writes one computes the normalisation itself)
-    for (int j = tid; j <= 2 * R; j += kCThreads) {
+    for (int j = tid; j < taps; j += kCThreads) {
+        if (j > 2 * R) {
+            wxy[j] = 0.f;
+            continue;  // loaded with its group, never used
+        }
         float s = 0.f;
         for (int q = -R; q <= R; ++q) s += (R == 0) ? 1.f : gauss_tap(q, g.sig_xy);
         wxy[j] = ((R == 0) ? 1.f : gauss_tap(j - R, g.sig_xy)) / s;
+        wdup[2 * j] = wdup[2 * j + 1] = wxy[j];
     }
     if (tid < W) {
         float s = 0.f;
@@ -88,28 +108,28 @@ __global__ void __launch_bounds__(kCThreads, (W <= 15 ? 2 : 1)) conv3d_tma_kerne
     __syncthreads();
 
     const uint32_t bytes = (uint32_t)(SY * BW * sizeof(float));
-    const int zbase = model * g.ez;
+    const int zbase = model * g.ez + k0;
     if (tid == 0) {
         tma_load_slab(&tmap, slab0, &bar[0], tx0, ty0, zbase, bytes);
-        if (g.ez > 1) tma_load_slab(&tmap, slab1, &bar[1], tx0, ty0, zbase + 1, bytes);
+        if (ne > 1) tma_load_slab(&tmap, slab1, &bar[1], tx0, ty0, zbase + 1, bytes);
     }
-    float wz[W];
+    f32x2 wz[W];
 #pragma unroll
-    for (int q = 0; q < W; ++q) wz[q] = s_wz[q];
+    for (int q = 0; q < W; ++q) wz[q] = pk2(s_wz[q], s_wz[q]);
 
-    // y-pass / z-pass ownership: column c, rows 4 gq .. 4 gq + 3
-    const int c = tid & 31, gq = tid >> 5;
-    float acc[4][W];
+    // y-pass / z-pass ownership: columns 2 c, 2 c + 1 (packed pairs), rows 2 gq, 2 gq + 1
+    const int c = tid & 15, gq = tid >> 4;
+    f32x2 acc[2][W];
 #pragma unroll
-    for (int p = 0; p < 4; ++p)
+    for (int p = 0; p < 2; ++p)
 #pragma unroll
-        for (int q = 0; q < W; ++q) acc[p][q] = 0.f;
+        for (int q = 0; q < W; ++q) acc[p][q] = pk2(0.f, 0.f);
     float *F = a.fine + (size_t)model * a.f_model_stride;
     const size_t fplane = (size_t)g.nyf * g.nxf;
-    const int ox = tx0 + c;
+    const int ox = tx0 + 2 * c;
     const int nitems = SY * (kCT / 4);  // x pass: (row, 4-column group)
 
-    for (int e = 0; e < g.ez; ++e) {
+    for (int e = 0; e < ne; ++e) {  // extended channel k0 + e
         float *slab = (e & 1) ? slab1 : slab0;
         if (!mbar_wait(&bar[e & 1], (uint32_t)((e >> 1) & 1), kWaitLimit)) {
             if (atomicExch(&s_abort, 1) == 0) atomicExch(&g_conv_status, 1);
@@ -118,64 +138,73 @@ __global__ void __launch_bounds__(kCThreads, (W <= 15 ? 2 : 1)) conv3d_tma_kerne
         if (s_abort) {
             // give the other buffer's copy, if one is in flight, a bounded
             // chance to land before the CTA leaves
-            if (tid == 0 && e + 1 < g.ez) mbar_wait(&bar[(e + 1) & 1], (uint32_t)(((e + 1) >> 1) & 1), kWaitLimit);
+            if (tid == 0 && e + 1 < ne) mbar_wait(&bar[(e + 1) & 1], (uint32_t)(((e + 1) >> 1) & 1), kWaitLimit);
             return;  // every thread sees the same flag after the barrier
         }
         // x pass: X[r][4 m .. 4 m + 3] from slab[r][4 m .. 4 m + 3 + 2R]
         for (int it = tid; it < nitems; it += kCThreads) {
             int r = it >> 3, m = it & 7;
-            const float *row = slab + r * BW + 4 * m;
+            const float4 *row = reinterpret_cast<const float4 *>(slab + r * BW + 4 * m);
             float o0 = 0.f, o1 = 0.f, o2 = 0.f, o3 = 0.f;
-            float v0 = row[0], v1 = row[1], v2 = row[2];
-            for (int j = 0; j <= 2 * R; ++j) {
-                float v3 = row[j + 3];
-                float w = wxy[j];
-                o0 = fmaf(w, v0, o0);
-                o1 = fmaf(w, v1, o1);
-                o2 = fmaf(w, v2, o2);
-                o3 = fmaf(w, v3, o3);
-                v0 = v1; v1 = v2; v2 = v3;
+            float4 p = row[0];
+            int j = 0;
+#pragma unroll 2
+            for (; j + 3 <= 2 * R; j += 4) {  // four taps per 16-byte load
+                const float4 n = row[j / 4 + 1], w = *reinterpret_cast<const float4 *>(wxy + j);
+                o0 = fmaf(w.x, p.x, o0); o1 = fmaf(w.x, p.y, o1); o2 = fmaf(w.x, p.z, o2); o3 = fmaf(w.x, p.w, o3);
+                o0 = fmaf(w.y, p.y, o0); o1 = fmaf(w.y, p.z, o1); o2 = fmaf(w.y, p.w, o2); o3 = fmaf(w.y, n.x, o3);
+                o0 = fmaf(w.z, p.z, o0); o1 = fmaf(w.z, p.w, o1); o2 = fmaf(w.z, n.x, o2); o3 = fmaf(w.z, n.y, o3);
+                o0 = fmaf(w.w, p.w, o0); o1 = fmaf(w.w, n.x, o1); o2 = fmaf(w.w, n.y, o2); o3 = fmaf(w.w, n.z, o3);
+                p = n;
+            }
+            {  // one tap (R even) or three (R odd) are left; BW is a multiple of 4, so the row holds n
+                const float4 w = *reinterpret_cast<const float4 *>(wxy + j);
+                o0 = fmaf(w.x, p.x, o0); o1 = fmaf(w.x, p.y, o1); o2 = fmaf(w.x, p.z, o2); o3 = fmaf(w.x, p.w, o3);
+                if (R & 1) {
+                    const float4 n = row[j / 4 + 1];
+                    o0 = fmaf(w.y, p.y, o0); o1 = fmaf(w.y, p.z, o1); o2 = fmaf(w.y, p.w, o2); o3 = fmaf(w.y, n.x, o3);
+                    o0 = fmaf(w.z, p.z, o0); o1 = fmaf(w.z, p.w, o1); o2 = fmaf(w.z, n.x, o2); o3 = fmaf(w.z, n.y, o3);
+                }
             }
             *reinterpret_cast<float4 *>(X + r * kCT + 4 * m) = make_float4(o0, o1, o2, o3);
         }
         __syncthreads();
         // the slab is consumed: refill it with channel e + 2
-        if (tid == 0 && e + 2 < g.ez) tma_load_slab(&tmap, slab, &bar[e & 1], tx0, ty0, zbase + e + 2, bytes);
-        // y pass: rows 4 gq .. 4 gq + 3 of column c
-        float y0 = 0.f, y1 = 0.f, y2 = 0.f, y3 = 0.f;
+        if (tid == 0 && e + 2 < ne) tma_load_slab(&tmap, slab, &bar[e & 1], tx0, ty0, zbase + e + 2, bytes);
+        // y pass: rows 2 gq, 2 gq + 1 of columns 2 c, 2 c + 1
+        f32x2 yv[2] = {pk2(0.f, 0.f), pk2(0.f, 0.f)};
         {
-            const float *col = X + (4 * gq) * kCT + c;
-            float v0 = col[0], v1 = col[kCT], v2 = col[2 * kCT];
+            const f32x2 *col = reinterpret_cast<const f32x2 *>(X + 2 * gq * kCT + 2 * c);
+            const f32x2 *w2 = reinterpret_cast<const f32x2 *>(wdup);
+            f32x2 v0 = col[0];
+#pragma unroll 4
             for (int j = 0; j <= 2 * R; ++j) {
-                float v3 = col[(j + 3) * kCT];
-                float w = wxy[j];
-                y0 = fmaf(w, v0, y0);
-                y1 = fmaf(w, v1, y1);
-                y2 = fmaf(w, v2, y2);
-                y3 = fmaf(w, v3, y3);
-                v0 = v1; v1 = v2; v2 = v3;
+                const f32x2 v1 = col[(j + 1) * (kCT / 2)];
+                yv[0] = fma2(w2[j], v0, yv[0]);
+                yv[1] = fma2(w2[j], v1, yv[1]);
+                v0 = v1;
             }
         }
-        // z pass: slot q holds output channel e - 2 Rz + q, weight wz[q]
-        float yv[4] = {y0, y1, y2, y3};
+        // z pass: slot q holds output channel e - 2 Rz + q, weight wz[q]; the
+        // sums move down one slot as they take the channel
+        const int k = k0 + e - 2 * Rz;
 #pragma unroll
-        for (int p = 0; p < 4; ++p) {
+        for (int p = 0; p < 2; ++p) {
+            const f32x2 out = fma2(wz[0], yv[p], acc[p][0]);
 #pragma unroll
-            for (int q = 0; q < W; ++q) acc[p][q] = fmaf(wz[q], yv[p], acc[p][q]);
-        }
-        int k = e - 2 * Rz;
-        if (k >= 0 && ox < g.nxf) {
-#pragma unroll
-            for (int p = 0; p < 4; ++p) {
-                int oy = ty0 + 4 * gq + p;
-                if (oy < g.nyf) F[(size_t)k * fplane + (size_t)oy * g.nxf + ox] = acc[p][0];
+            for (int q = 1; q < W; ++q) acc[p][q - 1] = fma2(wz[q], yv[p], acc[p][q]);
+            const int oy = ty0 + 2 * gq + p;
+            if (k >= k0 && ox < g.nxf && oy < g.nyf) {
+                float *dst = F + (size_t)k * fplane + (size_t)oy * g.nxf + ox;
+                if (a.vec2) {
+                    *reinterpret_cast<f32x2 *>(dst) = out;
+                } else {
+                    float lo, hi;
+                    upk2(out, lo, hi);
+                    dst[0] = lo;
+                    if (ox + 1 < g.nxf) dst[1] = hi;
+                }
             }
-        }
-#pragma unroll
-        for (int p = 0; p < 4; ++p) {
-#pragma unroll
-            for (int q = 0; q + 1 < W; ++q) acc[p][q] = acc[p][q + 1];
-            acc[p][W - 1] = 0.f;
         }
         // X is rewritten by the next x pass
         __syncthreads();
@@ -207,13 +236,13 @@ size_t conv_tma_smem_bytes(const Geom &g)
 {
     int SY = kCT + 2 * g.R, BW = (kCT + 2 * g.R + 3) & ~3;
     int SS = (SY * BW + 31) & ~31;
-    return 128 + sizeof(float) * (size_t)(2 * SS + SY * kCT + ((2 * g.R + 1 + 3) & ~3));
+    return 128 + sizeof(float) * (size_t)(2 * SS + SY * kCT + 3 * ((2 * g.R + 1 + 3) & ~3));
 }
 
 bool conv_tma_supported(const Geom &g)
 {
     int W = 2 * g.Rz + 1;
-    return W <= 23 && (kCT + 2 * g.R) <= 256 && conv_tma_smem_bytes(g) <= 200 * 1024 && encode_fn() != nullptr;
+    return W <= 23 && (kCT + 2 * g.R) <= 256 && conv_tma_smem_bytes(g) <= 200 * 1024 + 8 * (size_t)((2 * g.R + 1 + 3) & ~3) && encode_fn() != nullptr;
 }
 
 template <int W>
@@ -242,6 +271,7 @@ gbk_status launch_conv_tma(const StagedArgs &sa, cudaStream_t st)
     a.box_w = (kCT + 2 * g.R + 3) & ~3;
     a.fine = sa.fine;
     a.f_model_stride = sa.f_model_stride;
+    a.vec2 = g.nxf % 2 == 0 && sa.f_model_stride % 2 == 0 && reinterpret_cast<uintptr_t>(sa.fine) % 8 == 0;
     CUtensorMap tm;
     cuuint64_t dims[3] = {(cuuint64_t)sa.e_pitch, (cuuint64_t)g.ey, (cuuint64_t)g.ez * (cuuint64_t)sa.n_models};
     cuuint64_t strides[2] = {(cuuint64_t)sa.e_pitch * sizeof(float), (cuuint64_t)sa.e_pitch * g.ey * sizeof(float)};
@@ -252,7 +282,22 @@ gbk_status launch_conv_tma(const StagedArgs &sa, cudaStream_t st)
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return fail(GBK_ECUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
     size_t smem = conv_tma_smem_bytes(g);
-    int blocks = a.tiles_x * a.tiles_y * sa.n_models;
+    // ranges of channels: the count with the shortest queue of whole walks
+    const long tiles = (long)a.tiles_x * a.tiles_y * sa.n_models;
+    const long slots = 152 * (2 * g.Rz + 1 <= 15 && 2 * (smem + 1024) <= 228 * 1024 ? 2 : 1);
+    long best = 0;
+    a.zparts = 1;
+    a.zlen = g.nzf;
+    for (int z = 1; z <= 8 && z <= g.nzf; ++z) {
+        const int len = (g.nzf + z - 1) / z;
+        const long cost = ((tiles * z + slots - 1) / slots) * (len + 2 * g.Rz);
+        if (z == 1 || cost * 10 < best * 9) {  // a tenth better, for the channels read twice
+            best = cost;
+            a.zparts = (g.nzf + len - 1) / len;
+            a.zlen = len;
+        }
+    }
+    int blocks = (int)(tiles * a.zparts);
     switch (2 * g.Rz + 1) {
     case 1: return launch_w<1>(tm, a, smem, blocks, st);
     case 3: return launch_w<3>(tm, a, smem, blocks, st);
