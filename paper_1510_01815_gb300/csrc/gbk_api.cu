@@ -252,7 +252,17 @@ static gbk_status run_staged(const Geom &g, int32_t n, const double *params, flo
     a.partials = chi2 ? (double *)(base + L.off_part) : nullptr;
     if (obs) a.obs = *obs;
     bool want_moments = (maps || chi2 || resid);
-    gbk_status s = launch_staged(a, want_moments, st, ev);
+    gbk_status s;
+    if (!ev && cube_supported(g, n)) {
+        // the data cubes without the extended model cube's way through memory
+        // (its workspace stays a condition of the call); the timed stages
+        // are the chain's own
+        bool left = false;
+        if ((s = launch_cube(g, n, params, a.data, chi2 || resid ? nullptr : maps, st, &left))) return s;
+        if ((left || chi2 || resid) && (s = launch_moments(a, st))) return s;
+        return ok();
+    }
+    s = launch_staged(a, want_moments, st, ev);
     if (s) return s;
     return ok();
 }

@@ -43,9 +43,9 @@ __global__ void __launch_bounds__(256) model_cube_kernel(StagedArgs a)
     for (int q = 0; q < 4; ++q) {
         int xe = xe0 + q;
         float x = ((float)(xe - g.R) + 0.5f) * inv_u - 0.5f;
-        float br;
-        los(c, x, y, vl[q], br);
-        A[q] = (xe < g.ex && c.valid) ? c.amp * br : 0.f;
+        const float2 vb = line_at(c, x, y);
+        vl[q] = vb.x;
+        A[q] = (xe < g.ex && c.valid) ? c.amp * vb.y : 0.f;
         if (!c.valid) A[q] = __int_as_float(0x7fc00000);
     }
     float4 *out = reinterpret_cast<float4 *>(a.ext + (size_t)model * a.e_model_stride) + item;
@@ -165,22 +165,6 @@ __global__ void __launch_bounds__(256) downsample_kernel(StagedArgs a)
 // Moments of the data cube, one thread per spaxel.  Sums are taken about the
 // spaxel's own line-of-sight velocity clamped into the band, which keeps the
 // FP32 second moment free of cancellation.
-__device__ __forceinline__ void finish_moments(float s0, float s1, float s2, float cen,
-                                               const ModelConst &c, float &m0, float &m1, float &m2,
-                                               bool &valid)
-{
-    valid = s0 > kInvalidFraction * c.i0;
-    if (!c.valid) {
-        m0 = m1 = m2 = __int_as_float(0x7fc00000);
-    } else if (valid) {
-        float mu = s1 / s0;
-        m0 = s0;
-        m1 = cen + mu;
-        m2 = sqrtf(fmaxf(fmaf(-mu, mu, s2 / s0), 0.f));
-    } else {
-        m0 = 0.f; m1 = c.vsys; m2 = 0.f;
-    }
-}
 
 // Block sum of one FP32 value per thread: FP32 within each warp (a fixed
 // shuffle tree), the warps in FP64 in order.  Result in thread 0.
@@ -223,12 +207,9 @@ __global__ void __launch_bounds__(256) moments_kernel(StagedArgs a)
     float acc = 0.f;
     if (pix < np) {
         int y = pix / g.nx, x = pix - y * g.nx;
-        float vl, br;
-        los(c, (float)x, (float)y, vl, br);
-        // centre: v_los clamped into the band (see the fused kernel)
-        float cen = fminf(fmaxf(vl, g.vc - 0.5f * (float)(g.nz - 1) * g.dv), g.vc + 0.5f * (float)(g.nz - 1) * g.dv);
+        const float2 cb = moment_centre(c, g, (float)x, (float)y);
+        const float cen = cb.x, base = cb.y;
         const float *D = a.data + (size_t)model * a.d_model_stride + pix;
-        float base = g.vc - 0.5f * (float)(g.nz - 1) * g.dv - cen;
         float s0 = 0.f, s1 = 0.f, s2 = 0.f;
         // eight channel loads in flight per step; the sums stay in channel order
         int k = 0;
@@ -240,14 +221,14 @@ __global__ void __launch_bounds__(256) moments_kernel(StagedArgs a)
             for (int q = 0; q < 8; ++q) {
                 const float d = fmaf((float)(k + q), g.dv, base);
                 const float t = cv[q] * d;
-                s0 += cv[q]; s1 += t; s2 = fmaf(t, d, s2);
+                s0 += cv[q]; s1 = fmaf(cv[q], d, s1); s2 = fmaf(t, d, s2);
             }
         }
         for (; k < g.nz; ++k) {
             float cv = D[(size_t)k * np];
             float d = fmaf((float)k, g.dv, base);
             float t = cv * d;
-            s0 += cv; s1 += t; s2 = fmaf(t, d, s2);
+            s0 += cv; s1 = fmaf(cv, d, s1); s2 = fmaf(t, d, s2);
         }
         float m0, m1, m2;
         bool valid;
@@ -361,17 +342,22 @@ gbk_status launch_staged(const StagedArgs &a, bool want_moments, cudaStream_t st
         if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "down-sampling kernel launch");
     }
     if ((sm = mark(3))) return sm;
-    if (want_moments) {
-        int np = g.nx * g.ny;
-        int bpm = (np + 255) / 256;
-        moments_kernel<<<(unsigned)(bpm * a.n_models), 256, 0, stream>>>(a);
-        if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "moments kernel launch");
-        if (a.chi2) {
-            chi2_final_kernel<<<(a.n_models + 127) / 128, 128, 0, stream>>>(a.partials, bpm, a.n_models, a.chi2);
-            if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "chi2 final kernel launch");
-        }
-    }
+    if (want_moments && (sm = launch_moments(a, stream))) return sm;
     return mark(4);
+}
+
+gbk_status launch_moments(const StagedArgs &a, cudaStream_t stream)
+{
+    const int np = a.g.nx * a.g.ny;
+    const int bpm = (np + 255) / 256;
+    cudaError_t e;
+    moments_kernel<<<(unsigned)(bpm * a.n_models), 256, 0, stream>>>(a);
+    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "moments kernel launch");
+    if (a.chi2) {
+        chi2_final_kernel<<<(a.n_models + 127) / 128, 128, 0, stream>>>(a.partials, bpm, a.n_models, a.chi2);
+        if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "chi2 final kernel launch");
+    }
+    return GBK_OK;
 }
 
 cudaError_t launch_chi2_maps(int nx, int ny, int n_models, const float *maps, const gbk_obs &obs,
