@@ -1220,7 +1220,7 @@ def run_gbk(args):
                       "tuning": {"cluster_ctas": tuning["cluster_ctas"], "threads": tuning["threads"],
                                  "persistent": tuning["persistent"], "candidates": tuning["candidates"]},
                       "parallelism": "replicas" if ws > 1 else "single"},
-           "gpu_launches": K * (4 if staged else 1)}
+           "gpu_launches": K * (3 if staged else 1)}
     if split:
         # per-launch CUDA events (gbk_split_stage_times) over K further steps
         # of the same batches, L2 flushed before each: the kernels' times
@@ -1243,18 +1243,21 @@ def run_gbk(args):
 
     ex, ey, ez = ext_dims(g)
     if staged:
-        # HBM roofline of the staged chain: extended cube written and read
-        # once, data cube written and read once (algorithmic bytes)
+        # HBM roofline of the staged path: the data cube written by the cube
+        # kernel and read by the moments (algorithmic bytes; radii that this
+        # kernel does not serve also write and read the extended cube)
         peaks = {}
         try:
             peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))
         except Exception:
             pass
         hbm = float(peaks.get("hbm_gbs", 6800.0))
-        per_model = 4.0 * (2 * ex * ey * ez + 2 * g.nx * g.ny * g.nz)
+        one_kernel = g.upsample == 1 and ex - g.nx <= 16 and ez - g.nz <= 12
+        per_model = 4.0 * (2 * g.nx * g.ny * g.nz + (0 if one_kernel else 2 * ex * ey * ez))
         ach = n * per_model / (ms_step * 1e-3) / 1e9
         out["roofline"] = {"bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm,
-                           "traffic": None, "kernel": "staged chain (model cube, conv, moments)",
+                           "traffic": None, "kernel": "staged path (cube kernel, moments)" if one_kernel else
+                           "staged chain (model cube, conv, moments)",
                            "basis": "%.1f MB algorithmic traffic per model" % (per_model / 1e6),
                            "peak_source": "MEASURED_PEAKS.json hbm_gbs" if peaks else "fallback 6.8 TB/s"}
         # per-stage times (CUDA events between the stages, median of 5 calls

@@ -243,8 +243,9 @@ GBK_API gbk_status gbk_split_stage_times(const gbk_geom *g, int32_t n_models, co
                                          const gbk_obs *obs, double *chi2, void *workspace, size_t ws_bytes,
                                          float *stage_ms, int32_t *launches, void *stream);
 
-/* gbk_chi2 on the staged path (GBK_PATH_STAGED), timed per stage with CUDA
- * events on `stream` -- the per-step timings of the paper's GPU pipeline
+/* gbk_chi2 on the staged path (GBK_PATH_STAGED) as separate stages, timed with
+ * CUDA events on `stream` (gbk_chi2 itself takes the stages a1-a3 in one kernel
+ * where the radii allow it, with the same results) -- the per-step timings of the paper's GPU pipeline
  * (Sec. 5): stage_ms (host [4]) receives the milliseconds of the model cube
  * (a1-a2), the PSF x LSF convolution (a3), the down-sampling (a4; 0 at
  * u = 1) and the moments with the masked chi2 (a5-a6).  Workspace as for

@@ -1,6 +1,7 @@
-// fused_line.cuh -- the per-spaxel pieces of the folded forward model that
-// both fused evaluators use (k_fused.cu: one thread-block cluster per model;
-// k_split.cu: line sampling and PSF passes as separate stages).
+// fused_line.cuh -- the per-spaxel pieces of the folded forward model that the
+// evaluators and Jacobians share (k_fused.cu: one thread-block cluster per
+// model; k_tile.cu with line_table.cuh: one CTA per image or tile; k_tsplit.cu
+// and k_tangent.cu: the analytic Jacobians).
 //
 // Model: Bekiaris et al. 2015, Sec. 2.2.2 (cube), Sec. 2.1.7 / Eq. 9 and
 // Sec. 2.2.3 (PSF x LSF convolution), Sec. 2.2.5 (moments).  The identities
@@ -44,21 +45,6 @@ __device__ __forceinline__ void accum_shift(float4 q, float c, float w, float &s
     s1 += u;
     s2 = fmaf(w, q.z, s2);
     s2 = fmaf(D, u + t1, s2);
-}
-
-// Accumulates input (q0, q1, q2 about a; l1 = q1 + a q0, h1 = 2 q1
-// precomputed per input) into output sums with weight w: s0 and s1 about 0,
-// s2 about the output's centre c, exactly re-centred (D = a - c): six FP32
-// operations.  The caller moves s1 to c once at the end (s1 - c s0).
-__device__ __forceinline__ void accum_lin(float q0, float l1, float h1, float q2, float a, float c, float w,
-                                          float &s0, float &s1, float &s2)
-{
-    const float D = a - c;
-    s0 = fmaf(w, q0, s0);
-    s1 = fmaf(w, l1, s1);
-    const float i1 = fmaf(D, q0, h1);
-    const float i2 = fmaf(D, i1, q2);
-    s2 = fmaf(w, i2, s2);
 }
 
 // An input (q0, q1, q2 about its centre a) moved exactly to a reference

@@ -25,7 +25,7 @@
 // (zparts), whose moments then take moments_kernel's pass over the cube.
 //
 // 256 models of 64 x 64 x 64 (R = 5, Rz = 3): 284 us by the staged chain (1.3
-// GB moved), 178 us here (268 MB).
+// GB moved), 176 us here (268 MB).
 // The packed FMAs (two passes of the FMA pipe each, busy 60 %) and their issue
 // slots (63 %) bound it; 31 models of 142 x 128 x 102: 256 -> 159 us, 4 models
 // of 64 x 25 x 74: 62 -> 23 us.

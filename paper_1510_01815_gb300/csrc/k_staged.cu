@@ -12,6 +12,8 @@
 //                       partials (Sec. 2.2.5-2.2.6)
 //   chi2_final_kernel   fixed-order FP64 sum of the partials
 //   chi2_maps_kernel    Eq. 11 from caller-supplied maps, one block per model
+//
+// At u = 1 and small radii k_cube.cu writes the data cube without the first two.
 #include "gbk_api_internal.h"
 #include "gbk_internal.cuh"
 #include "k_staged.h"

@@ -1,6 +1,6 @@
 // tma_util.cuh -- shared-memory addresses, mbarriers with bounded waits and
 // 3-D TMA tile loads used by the staged convolution kernels and the split
-// evaluator's PSF stage.
+// Jacobian's PSF stage.
 #pragma once
 
 #include <cuda.h>
