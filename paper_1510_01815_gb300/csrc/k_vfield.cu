@@ -96,6 +96,7 @@ __global__ void __cluster_dims__(kVfRanks, 1, 1) __launch_bounds__(kVfThreads) v
     const int mpg = a.models_per_gal;
     const int first = rank * 32 + lane;  // the chain's first pixel
     const float nanf_ = __int_as_float(0x7fc00000);
+    cluster.sync();  // every CTA has started: its shared memory may be written
     for (int model = blockIdx.x / kVfRanks; model < a.n_models; model += gridDim.x / kVfRanks) {
         const int gal = mpg > 0 ? model / mpg : 0;
         if (a.skip && a.skip[gal] != 0) continue;  // the whole cluster
@@ -234,6 +235,7 @@ __global__ void __cluster_dims__(kVfRanks, 1, 1) __launch_bounds__(kVfThreads) v
     const int mpg = a.models_per_gal;
     const int first = rank * 32 + lane;  // the chain's first pixel
     const float kdeg = 0.017453292519943295f;
+    cluster.sync();  // every CTA has started: its shared memory may be written
     for (int model = blockIdx.x / kVfRanks; model < a.n_models; model += gridDim.x / kVfRanks) {
         const int gal = mpg > 0 ? model / mpg : 0;
         if (a.skip && a.skip[gal] != 0) continue;  // the whole cluster
