@@ -57,15 +57,18 @@ struct CnnTables {
     size_t off[kCnnL + 1];
     __nv_bfloat16 *W[kCnnL], *WT[kCnnL];
     float *bias[kCnnL];
-    __nv_bfloat16 *W0q;  // the first layer's weights four times, block-diagonal [4 C_0][4 K_0]
+    __nv_bfloat16 *W0q;  // the first layer's weights four times side by side [C_0][4 K_0]
     float *bias0q;       // and its biases four times
 };
 
-// The first layer runs on four rows at a time: its patch matrix [M][16] read
-// as [M / 4][64] against four copies of the weights on the diagonal is the
-// same product (the added terms are exact zeros) with full 128-byte rows for
-// the tensor copies; as 32-byte rows of a 64-wide box, most of it fill, they
-// set the time (1048576 x 32 x 16 with one epilogue: 102 us, so 78 us).
+// The first layer runs on four rows at a time: its patch matrix [M][16] is
+// read as [M / 4][64], with full 128-byte rows for the tensor copies; as
+// 32-byte rows of a 64-wide box, most of it fill, they set the time (1048576 x
+// 32 x 16 with one epilogue: 102 us, so 78 us).  Each of the four has its own
+// instruction and columns of the accumulator (GemmArgs::fours), so a patch
+// with a NaN or an infinity stays alone with it: against four copies of the
+// weights on the diagonal of one operand, the three other rows took it times
+// zero.
 constexpr int kCnnQ = 4;
 
 __device__ __forceinline__ uint64_t sm_mix(uint64_t z)
@@ -145,9 +148,7 @@ __global__ void cnn_publish_kernel(const float *P, CnnTables t, bool backward, C
             const __nv_bfloat16 h = __float2bfloat16_rn(v);
             t.W[l][(size_t)o * K + k] = h;
             if (l == 0)
-                for (unsigned q = 0; q < kCnnQ; ++q)
-                    for (unsigned p = 0; p < kCnnQ; ++p)
-                        t.W0q[(size_t)(q * C + o) * (kCnnQ * K) + p * K + k] = p == q ? h : __float2bfloat16_rn(0.f);
+                for (unsigned q = 0; q < kCnnQ; ++q) t.W0q[(o * kCnnQ + q) * K + k] = h;
             if (backward) t.WT[l][(size_t)k * C + o] = h;
         }
     }
@@ -390,7 +391,7 @@ static CnnWs cnn_layout(int B, char *base)
         w.t.bias[l] = (float *)take(sizeof(float) * kCnnC[l]);
     }
     w.t.off[kCnnL] = param_count();
-    w.t.W0q = (__nv_bfloat16 *)take(bf * kCnnQ * kCnnC[0] * kCnnQ * kCnnK[0]);
+    w.t.W0q = (__nv_bfloat16 *)take(bf * kCnnC[0] * kCnnQ * kCnnK[0]);
     w.t.bias0q = (float *)take(sizeof(float) * kCnnQ * kCnnC[0]);
     w.total = o;
     return w;
@@ -447,6 +448,7 @@ static gbk_status cnn_forward_ws(const CnnWs &w, int B, bool want_transposed, cu
             a.ldo *= kCnnQ;
             a.bias = w.t.bias0q;
             a.t_log2 = 0;
+            a.fours = 1;
             W = w.t.W0q;
         }
         if ((s = gemm(w.A[l], a.K, W, a.K, a, st))) return s;

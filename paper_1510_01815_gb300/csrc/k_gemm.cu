@@ -35,6 +35,7 @@
 namespace gbk {
 
 constexpr int kGBM = 128, kGBK = 64, kGMaxStages = 8, kGThreads = 192, kGGroup = 16;
+constexpr int kGFour = 32;  // columns of a part of GemmArgs::fours
 constexpr int kGMaxCtas = 3;  // CTAs per SM at most (113 registers a thread)
 // Bounded waits: 2^18 try_wait attempts, about one second (a try that finds
 // its phase incomplete suspends about 3.75 us on GB300, as gbk_wait_selfcheck
@@ -295,7 +296,8 @@ __device__ __forceinline__ void gemm_epilogue_quad(const GemmArgs &a, float *out
 }
 
 // CTAS: CTAs that share an SM (registers: 256-column tiles run alone on it).
-template <int CTAS>
+// FOURS: GemmArgs::fours.
+template <int CTAS, bool FOURS>
 __global__ void __launch_bounds__(kGThreads, CTAS)
     gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, GemmArgs a,
                      int units)
@@ -304,14 +306,15 @@ __global__ void __launch_bounds__(kGThreads, CTAS)
     const int tiles_m = (a.M + kGBM - 1) / kGBM, tiles_n = (a.N + BN - 1) / BN;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int KT_all = (a.K + kGBK - 1) / kGBK;
-    const uint32_t bytesA = kGBM * kGBK * 2, bytesB = (uint32_t)BN * kGBK * 2;
+    const int brows = FOURS ? kGFour : BN;  // rows of B in a slab
+    const uint32_t bytesA = kGBM * kGBK * 2, bytesB = (uint32_t)brows * kGBK * 2;
 
     extern __shared__ __align__(1024) unsigned char gsm_raw[];
     // 128-byte swizzled tiles must start on 1024-byte boundaries
     unsigned char *gsm = gsm_raw + ((1024u - (g_smem_u32(gsm_raw) & 1023u)) & 1023u);
     unsigned char *sA = gsm;                      // [stages][128][64] bf16
     const int stages = a.stages;
-    unsigned char *sB = gsm + stages * bytesA;  // [stages][BN][64] bf16
+    unsigned char *sB = gsm + stages * bytesA;  // [stages][brows][64] bf16
     __shared__ __align__(8) uint64_t full[kGMaxStages], empty[kGMaxStages], acc_full[2], acc_empty[2];
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
@@ -359,7 +362,7 @@ __global__ void __launch_bounds__(kGThreads, CTAS)
                                  "r"(bytesA + bytesB)
                                  : "memory");
                     g_tma_2d(&tmA, sA + (size_t)s * bytesA, &full[s], (t.kt0 + kt) * kGBK, t.m0);
-                    g_tma_2d(&tmB, sB + (size_t)s * bytesB, &full[s], (t.kt0 + kt) * kGBK, t.n0);
+                    g_tma_2d(&tmB, sB + (size_t)s * bytesB, &full[s], (t.kt0 + kt) * kGBK, FOURS ? 0 : t.n0);
                     if (++s == stages) {
                         s = 0;
                         ph ^= 1u;
@@ -371,7 +374,7 @@ __global__ void __launch_bounds__(kGThreads, CTAS)
     } else if (warp == 1) {
         if (lane == 0) {
             // MMA issuer: tile i accumulates into buffer i % 2
-            const uint32_t idesc = idesc_bf16_f32(kGBM, BN);
+            const uint32_t idesc = idesc_bf16_f32(kGBM, brows);
             int s = 0;
             uint32_t ph = 0;
             bool go = true;
@@ -392,15 +395,29 @@ __global__ void __launch_bounds__(kGThreads, CTAS)
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint64_t da = smem_desc_k128(g_smem_u32(sA + (size_t)s * bytesA));
                     const uint64_t db = smem_desc_k128(g_smem_u32(sB + (size_t)s * bytesB));
+                    if constexpr (FOURS) {
+                        // the slab's k-th 16 columns of A are rows of their
+                        // own: each into its own columns of the accumulator
+#pragma unroll 1
+                        for (int c = 0; c < BN; c += kGFour) {
+                            const uint64_t k = (uint64_t)(2 * ((t.n0 + c) / kGFour));
+                            asm volatile(
+                                "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                                " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtm + (uint32_t)c),
+                                "l"(da + k), "l"(db + k), "r"(idesc), "r"(0u)
+                                : "memory");
+                        }
+                    } else {
 #pragma unroll
-                    for (int kk = 0; kk < kGBK / 16; ++kk) {
-                        // advance 16 elements (32 B) along K inside the swizzle atom
-                        const uint32_t acc = (kt > 0 || kk > 0) ? 1u : 0u;
-                        asm volatile(
-                            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtm),
-                            "l"(da + (uint64_t)(2 * kk)), "l"(db + (uint64_t)(2 * kk)), "r"(idesc), "r"(acc)
-                            : "memory");
+                        for (int kk = 0; kk < kGBK / 16; ++kk) {
+                            // advance 16 elements (32 B) along K inside the swizzle atom
+                            const uint32_t acc = (kt > 0 || kk > 0) ? 1u : 0u;
+                            asm volatile(
+                                "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                                " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtm),
+                                "l"(da + (uint64_t)(2 * kk)), "l"(db + (uint64_t)(2 * kk)), "r"(idesc), "r"(acc)
+                                : "memory");
+                        }
                     }
                     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                                      g_smem_u32(&empty[s]))
@@ -543,6 +560,8 @@ gbk_status launch_gemm_bf16(const void *A, int lda, const void *B, int ldb, cons
     if (((uintptr_t)A % 16) || ((uintptr_t)B % 16)) return fail(GBK_EINVAL, "A and B must be 16-byte aligned");
     if (a.ldo < a.N) return fail(GBK_EINVAL, "ldo must be >= N");
     if (!a.out_bf16 && !a.out_f32) return fail(GBK_EINVAL, "no output");
+    if (a.fours && (a.K != kGBK || a.N != 4 * kGFour || a.kt_split > 0))
+        return fail(GBK_EINVAL, "rows in fours need K = 64 and four parts of 32 columns");
     a.bn = a.N >= 256 ? 256 : (a.N >= 128 ? 128 : ((a.N + 15) / 16) * 16);
     // Tiles for less than half the SMs: narrower ones, so that more SMs share
     // the loads and the epilogue (1024 x 256 x 4096, the network's first dense
@@ -568,12 +587,14 @@ gbk_status launch_gemm_bf16(const void *A, int lda, const void *B, int ldb, cons
     CUtensorMap ta, tb;
     gbk_status s = encode_kmajor(&ta, A, a.M, a.K, lda, kGBM);
     if (s) return s;
-    if ((s = encode_kmajor(&tb, B, a.N, a.K, ldb, a.bn))) return s;
+    if ((s = encode_kmajor(&tb, B, a.fours ? kGFour : a.N, a.K, ldb, a.fours ? kGFour : a.bn))) return s;
     size_t smem = gemm_smem_bytes(a.bn, a.stages);
     const int ctas = std::max(1, std::min(kGMaxCtas, gemm_per_sm(a.bn, a.stages)));
-    auto *const kernel = ctas > 1 ? &gemm_bf16_kernel<kGMaxCtas> : &gemm_bf16_kernel<1>;
-    static KernelAttrMemo memo1, memo3;
-    if ((s = ensure_kernel_attrs((const void *)kernel, smem, false, ctas > 1 ? memo3 : memo1,
+    auto *const kernel = a.fours    ? &gemm_bf16_kernel<kGMaxCtas, true>
+                         : ctas > 1 ? &gemm_bf16_kernel<kGMaxCtas, false>
+                                    : &gemm_bf16_kernel<1, false>;
+    static KernelAttrMemo memo1, memo3, memo4;
+    if ((s = ensure_kernel_attrs((const void *)kernel, smem, false, a.fours ? memo4 : (ctas > 1 ? memo3 : memo1),
                                  "GEMM: setting dynamic shared memory")))
         return s;
     int splits = 1;

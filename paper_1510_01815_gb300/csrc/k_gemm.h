@@ -30,6 +30,11 @@ struct GemmArgs {
     // the FP32 slice out_f32 + z * split_stride (0: no split).
     int kt_split;
     size_t split_stride;
+    // Rows of A in fours: A [M][64] holds four rows of 16 each, B [32][64] the
+    // weights [32][16] four times side by side (full rows: copies that fill
+    // most of a box with zeros are slow), and output columns 32 q .. 32 q + 31
+    // are the product of the q-th (K = 64, N = 128, no split).
+    int fours;
 };
 
 gbk_status launch_gemm_bf16(const void *A, int lda, const void *B, int ldb, const GemmArgs &args, cudaStream_t st);
