@@ -66,6 +66,11 @@ struct LineTab {
     float inv_dv;
 };
 
+// 1 / the unit of length of los_disc2: r_t held to [1e-12, 1e9] pixels.
+// Below, atan(r / r_t) is pi/2 at every FP32 position but the centre itself;
+// above, atan(u) / u is 1 and disc_const's k carries the rest.
+__device__ __forceinline__ float disc_inv_unit(const ModelConst &c) { return fminf(fmaxf(c.inv_rt, 1e-9f), 1e12f); }
+
 // The forms that serve a model (the same whatever the tiling, so are the
 // sums).  A few dozen operations: one thread computes it for its block.
 __device__ inline LineTab line_table_plan(const Geom &g, const ModelConst &c, const LineCtx &L)
@@ -76,6 +81,12 @@ __device__ inline LineTab line_table_plan(const Geom &g, const ModelConst &c, co
     T.c1 = -1.f;
     const float s = c.sigma;
     if (!c.valid || !(s >= kLtNarrow * g.dv)) return T;
+    // los_disc2 squares lengths in units of r_t: where the farthest deprojected
+    // one might overflow (r_t = 1e-12 px under more than 89.999 degrees, a
+    // centre far outside the image) every spaxel takes the direct sum, whose
+    // lengths are in pixels.
+    const float far = (float)(g.ex + g.ey) + fabsf(c.x0) + fabsf(c.y0);
+    if (!(far * c.inv_cos_i * disc_inv_unit(c) < 1e18f)) return T;
     const float B = L.v_hi - L.v_lo;
     if (B > 0.f) {
         const float nb = ceilf(B / (kLtWidth * s));
@@ -271,7 +282,8 @@ __device__ __forceinline__ void line_closed(const LineTab &T, float vz0, float v
 // rows in the lanes of f32x2 operations.  Lengths are in units of r_t, so
 // with u = r / r_t the velocity is Vsys + (2/pi) Vmax sin i (x_e / r_t)
 // atan(u) / u: atan(s) / s is a polynomial in s^2 on [0, 1] (minimax in
-// relative error, 2e-9, found by a Remez exchange), taken at s = u, or at
+// relative error found by a Remez exchange; 5e-9 with its constants rounded
+// to FP32), taken at s = u, or at
 // s = 1/u with atan(u) = pi/2 - atan(1/u); both u and 1/u come from one
 // reciprocal square root, and no division is left.
 struct DiscConst {
@@ -283,10 +295,7 @@ __device__ __forceinline__ f32x2 dup2(float v) { return pk2(v, v); }
 
 __device__ __forceinline__ DiscConst disc_const(const ModelConst &c)
 {
-    // The unit of length is r_t held to [1e-12, 1e9] pixels, so that u^2
-    // stays in range: below, atan(r / r_t) is pi/2 at every FP32 position but
-    // the centre itself; above, atan(u) / u is 1 and k carries the rest.
-    const float ir = fminf(fmaxf(c.inv_rt, 1e-9f), 1e12f);
+    const float ir = disc_inv_unit(c);
     DiscConst d;
     d.x0 = c.x0;
     d.y0 = c.y0;
