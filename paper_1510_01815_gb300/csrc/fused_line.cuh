@@ -196,8 +196,11 @@ __device__ __forceinline__ void los_line(const ModelConst &c, float x, float y, 
 // in the band, <= kUFlush for one centred outside it, one channel of margin),
 // two channels per packed FP32 instruction, stepping u by additions that are
 // re-anchored by one FMA every six channel pairs.
-// Must be called by whole warps (the lanes of a warp share the channel
-// window); inactive lanes are allowed.
+// WARP: called by whole warps (the lanes of a warp share the channel window;
+// inactive lanes are allowed).  Without it each lane takes its own window: for
+// calls that only some lanes make, whose sums would otherwise depend on which
+// lanes those are.
+template <bool WARP>
 __device__ __forceinline__ float4 line_sums(const Geom &g, const ModelConst &c, const LineCtx &L,
                                             const float *eG0, const float *eA1, const float *eA2, float x, float y)
 {
@@ -213,16 +216,16 @@ __device__ __forceinline__ float4 line_sums(const Geom &g, const ModelConst &c, 
     const float sh = vl - a_c;
     const float ub = L.al * (L.vz0 - vl);  // u = alpha (v_e - v_los) at e = 0
     const f32x2 UB = pk2(ub, ub);
-    const unsigned am = __activemask();
-    const bool outside = __any_sync(am, sh != 0.f);
+    const unsigned am = WARP ? __activemask() : 0u;
+    const bool outside = WARP ? __any_sync(am, sh != 0.f) : true;  // alone: one form for all lanes
 
-    // channel window of the warp: the union of the lanes' |u| <= cut
+    // channel window: |u| <= cut (WARP: the union of the lanes')
     const float cut = (sh != 0.f) ? kUFlush : kUCut;
     float flo = (-cut - ub) * L.inv_adv - 1.f, fhi = (cut - ub) * L.inv_adv + 1.f;
     if (!(flo > -1e6f)) flo = -1e6f;
     if (!(fhi < 1e6f)) fhi = 1e6f;
-    const int wlo = __reduce_min_sync(am, (int)floorf(flo));
-    const int whi = __reduce_max_sync(am, (int)ceilf(fhi));
+    const int wlo = WARP ? __reduce_min_sync(am, (int)floorf(flo)) : (int)floorf(flo);
+    const int whi = WARP ? __reduce_max_sync(am, (int)ceilf(fhi)) : (int)ceilf(fhi);
 
     // interior channels [elo, ehi): sums of g, g m, g m^2 with m = alpha (v_e - a)
     int e = L.elo, e_stop = L.ehi;
@@ -255,7 +258,7 @@ __device__ __forceinline__ float4 line_sums(const Geom &g, const ModelConst &c, 
             U = add2(U, ADV2);
         }
     } else {
-        // some lane of the warp has its line outside the band: m = u + alpha sh
+        // a line outside the band: m = u + alpha sh
         const float su = L.al * sh;
         const f32x2 SU = pk2(su, su);
         for (; e + 12 <= e_stop; e += 12) {
@@ -268,7 +271,7 @@ __device__ __forceinline__ float4 line_sums(const Geom &g, const ModelConst &c, 
                 const f32x2 G = pk2(ex2_approx(-w0), ex2_approx(-w1));
                 const f32x2 M = add2(U, SU);
                 const f32x2 T = mul2(G, M);
-                S0 = add2(S0, G); S1 = add2(S1, T); S2 = fma2(T, M, S2);
+                S0 = add2(S0, G); S1 = WARP ? add2(S1, T) : fma2(G, M, S1); S2 = fma2(T, M, S2);
                 U = add2(U, ADV2);
             }
             FE = add2(FE, TWELVE);
@@ -281,7 +284,7 @@ __device__ __forceinline__ float4 line_sums(const Geom &g, const ModelConst &c, 
             const f32x2 G = pk2(ex2_approx(-w0), ex2_approx(-w1));
             const f32x2 M = add2(U, SU);
             const f32x2 T = mul2(G, M);
-            S0 = add2(S0, G); S1 = add2(S1, T); S2 = fma2(T, M, S2);
+            S0 = add2(S0, G); S1 = WARP ? add2(S1, T) : fma2(G, M, S1); S2 = fma2(T, M, S2);
             U = add2(U, ADV2);
         }
     }
@@ -296,7 +299,7 @@ __device__ __forceinline__ float4 line_sums(const Geom &g, const ModelConst &c, 
     float q0 = s0, q1 = s1 * L.inv_al, q2 = fmaf(s2, L.inv_al * L.inv_al, L.var_z * s0);
 
     // edge blocks: E0 = sum g G0, B1 = sum g A1, B2 = sum g A2 over the part
-    // of the block inside the warp's window
+    // of the block inside the window
     for (int blk = 0; blk < 2; ++blk) {
         int eb = blk ? L.ehi : 0, ee = blk ? g.ez : L.elo;
         if (wlo > eb) eb += (min(wlo, ee) - eb) & ~1;  // an even offset keeps the table pairs aligned

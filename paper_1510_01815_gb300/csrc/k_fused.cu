@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(NT, MINB) fused_eval_kernel(FusedArgs a)
     const int dr_e = nthr / g.ex, dx_e = nthr - dr_e * g.ex;  // (row, col) step of idx += nthr
     for (int idx = tid; idx < nsp; idx += nthr) {
         const float x = (float)(xe - R), y = (float)(row0 + r - R);
-        Q[idx] = line_sums(g, c, lc, eG0, eA1, eA2, x, y);
+        Q[idx] = line_sums<true>(g, c, lc, eG0, eA1, eA2, x, y);
         xe += dx_e; r += dr_e;
         if (xe >= g.ex) { xe -= g.ex; ++r; }
     }

@@ -263,24 +263,57 @@ __device__ __forceinline__ void psf_pass(const Load &load, uint32_t taps, f32x2 
 }
 
 // The lines of the extended tile; task: column x of a row pair, two spaxels.
+// Spaxels that neither form serves are marked with NaN and their threads come
+// back to them in a loop of their own for the direct sum: as a call from the
+// first loop it cost every model registers, and warps that took it for single
+// lanes up to half of the models' time where all lines lie outside the band.
+// Each lane of it has its own channel window; shared by the lanes that happen
+// to be there, it made the last bits depend on the tiling.
 __device__ __forceinline__ void lines_phase(const Geom &g, const TileItem &M, int R, const float *edge,
                                             const float *ltab, float *pl, int tid, int nthr)
 {
-    const int etl = edge_table_len(g);
     const int exw = M.d.exw, PP = M.d.PP, RP = M.d.RP, ntl = M.d.nrp * exw;
-    const DiscConst dc = disc_const(M.mc);
-    int x, rp, dx, drp;
-    split_index(tid, exw, rp, x);
+    int x0, rp0, dx, drp;
+    split_index(tid, exw, rp0, x0);
     split_index(nthr, exw, drp, dx);
     const float xb = (float)(M.d.tx0 - R), yb = (float)(M.d.ty0 - R);
+    const bool all = line_table_empty(M.lt);
+    bool left = all;
+    if (!all) {
+        const DiscConst dc = disc_const(M.mc);
+        int x = x0, rp = rp0;
+        for (int idx = tid; idx < ntl; idx += nthr) {
+            float4 q[2];
+            line_sums_pair(dc, M.lc, M.lt, ltab, xb + (float)x, yb + (float)(2 * rp), q, left);
+            float *o = pl + rp * RP + 2 * x;
+            *reinterpret_cast<float2 *>(o) = make_float2(q[0].x, q[1].x);
+            *reinterpret_cast<float2 *>(o + PP) = make_float2(q[0].y, q[1].y);
+            *reinterpret_cast<float2 *>(o + 2 * PP) = make_float2(q[0].z, q[1].z);
+            *reinterpret_cast<float2 *>(o + 3 * PP) = make_float2(q[0].w, q[1].w);
+            x += dx;
+            rp += drp;
+            if (x >= exw) {
+                x -= exw;
+                ++rp;
+            }
+        }
+    }
+    if (!left) return;
+    const int etl = edge_table_len(g);
+    const float inv_i0 = 1.f / M.mc.i0;
+    int x = x0, rp = rp0;
     for (int idx = tid; idx < ntl; idx += nthr) {
-        float4 q[2];
-        line_sums_pair(g, M.mc, dc, M.lc, M.lt, ltab, edge, etl, xb + (float)x, yb + (float)(2 * rp), q);
-        float *o = pl + rp * RP + 2 * x;
-        *reinterpret_cast<float2 *>(o) = make_float2(q[0].x, q[1].x);
-        *reinterpret_cast<float2 *>(o + PP) = make_float2(q[0].y, q[1].y);
-        *reinterpret_cast<float2 *>(o + 2 * PP) = make_float2(q[0].z, q[1].z);
-        *reinterpret_cast<float2 *>(o + 3 * PP) = make_float2(q[0].w, q[1].w);
+        float *const o = pl + rp * RP + 2 * x;
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            if (!all && !isnan(o[h])) continue;
+            const float4 q = line_sums<false>(g, M.mc, M.lc, edge, edge + etl, edge + 2 * etl, xb + (float)x,
+                                              yb + (float)(2 * rp + h));
+            o[h] = q.x * inv_i0;
+            o[PP + h] = q.y * inv_i0;
+            o[2 * PP + h] = q.z * inv_i0;
+            o[3 * PP + h] = q.w;
+        }
         x += dx;
         rp += drp;
         if (x >= exw) {

@@ -239,6 +239,9 @@ __device__ inline void line_table_build(const Geom &g, const LineCtx &L, const L
     __syncthreads();
 }
 
+// Neither form serves any of the model's lines.
+__device__ __forceinline__ bool line_table_empty(const LineTab &T) { return T.nseg == 0 && T.c0 > T.c1; }
+
 // The polynomials' sums (q0, q1, q2) at position t of a stored segment.
 __device__ __forceinline__ void line_table_eval(const float *tab, int seg, float t, float &q0, float &q1, float &q2)
 {
@@ -361,21 +364,13 @@ __device__ __forceinline__ void los_disc2(const DiscConst &d, float x, float y, 
     A1 = d.A * ex2_approx(d.hl * ub);
 }
 
-// The direct sum of the few spaxels that the forms above do not serve, out
-// of line: its registers stay out of the caller's loop.
-static __device__ __noinline__ float4 line_sums_direct(const Geom *g, const ModelConst *c, const LineCtx *L,
-                                                       const float *edge, int etl, float x, float y)
+// The line sums of a spaxel with velocity v that the closed form does not
+// serve (per unit amplitude); NaN in q.x, and `left` set, where the polynomials
+// do not either.
+__device__ __forceinline__ float4 line_sums_edge(const LineCtx &L, const LineTab &T, const float *tab, float v,
+                                                 bool &left)
 {
-    return line_sums(*g, *c, *L, edge, edge + etl, edge + 2 * etl, x, y);
-}
-
-// The line sums of a spaxel at (x, y) with velocity v that the closed form
-// does not serve (per unit amplitude); `edge` holds the three edge tables of
-// etl floats each.  False: q holds the direct sum, amplitude included.
-__device__ __forceinline__ bool line_sums_edge(const Geom &g, const ModelConst &c, const LineCtx &L, const LineTab &T,
-                                               const float *tab, const float *edge, int etl, float x, float y,
-                                               float v, float4 &q)
-{
+    float4 q;
     const float p = (v - T.v0) * T.inv_w, fl = floorf(p);
     const int seg = (int)fl, lows = T.int0 - T.first, gap = T.int1 - T.int0;
     // a velocity just inside the closed form's outermost segments belongs to
@@ -393,19 +388,20 @@ __device__ __forceinline__ bool line_sums_edge(const Geom &g, const ModelConst &
         st = lows;
         t -= 2.f * (float)(lows + gap - seg);
     }
-    if (!(p >= 0.f && st >= 0 && st < T.nseg)) {
-        q = line_sums_direct(&g, &c, &L, edge, etl, x, y);
-        return false;
+    if (p >= 0.f && st >= 0 && st < T.nseg) {
+        line_table_eval(tab, st, t, q.x, q.y, q.z);
+    } else {
+        q.x = q.y = q.z = __int_as_float(0x7fc00000);
+        left = true;
     }
-    line_table_eval(tab, st, t, q.x, q.y, q.z);
     q.w = fminf(fmaxf(v, L.v_lo), L.v_hi);
-    return true;
+    return q;
 }
 
-// The line sums (A q0, A q1, A q2, a) of the spaxels at (x, y) and (x, y + 1).
-__device__ __forceinline__ void line_sums_pair(const Geom &g, const ModelConst &c, const DiscConst &d, const LineCtx &L,
-                                               const LineTab &T, const float *tab, const float *edge, int etl, float x,
-                                               float y, float4 (&q)[2])
+// The line sums (A q0, A q1, A q2, a) of the spaxels at (x, y) and (x, y + 1),
+// per unit I0; NaN in q[h].x, and `left` set, where only the direct sum serves.
+__device__ __forceinline__ void line_sums_pair(const DiscConst &d, const LineCtx &L, const LineTab &T,
+                                               const float *tab, float x, float y, float4 (&q)[2], bool &left)
 {
     float v[2], A[2];
     los_disc2(d, x, y, v[0], v[1], A[0], A[1]);
@@ -414,8 +410,8 @@ __device__ __forceinline__ void line_sums_pair(const Geom &g, const ModelConst &
         if (v[h] >= T.c0 && v[h] <= T.c1) {
             line_closed(T, L.vz0, v[h], q[h].x, q[h].y, q[h].z);
             q[h].w = v[h];
-        } else if (!line_sums_edge(g, c, L, T, tab, edge, etl, x, y + (float)h, v[h], q[h])) {
-            A[h] = 1.f / c.i0;
+        } else {
+            q[h] = line_sums_edge(L, T, tab, v[h], left);
         }
         q[h].x *= A[h];
         q[h].y *= A[h];
