@@ -411,6 +411,10 @@ __device__ __forceinline__ float y_phase(const TileItem &M, uint32_t taps, const
             upk2(cen, ce[0], ce[1]);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
+                // __frcp_rn and sqrtf here cost 7 - 9 % of the whole call
+                // (8192 images of 64 x 64: 482 -> 527 us) and move the
+                // dispersion's error against 64 bits from 0.94 to 0.92 of what
+                // it was with sampled lines, so the approximations stay
                 valid[h] = s0[h] > kInvalidFraction;
                 const float inv = rcp_approx(s0[h]), mu = s1[h] * inv;
                 const float var = fmaf(-mu, mu, s2[h] * inv);

@@ -288,7 +288,10 @@ __device__ __forceinline__ void line_closed(const LineTab &T, float vz0, float v
 // relative error found by a Remez exchange; 5e-9 with its constants rounded
 // to FP32), taken at s = u, or at
 // s = 1/u with atan(u) = pi/2 - atan(1/u); both u and 1/u come from one
-// reciprocal square root, and no division is left.
+// reciprocal square root, and no division is left.  One Newton step refines
+// both: over 46 cases of the declared ranges the velocity maps' error against
+// 64 bits is then 1.01 times that of a square root and a division, 1.02 times
+// with 1/u as the instruction gives it; the step's time does not show.
 struct DiscConst {
     float x0, y0, a1, a2, b1, b2;  // x_e / r_t = a1 dx + a2 dy, -y_e / (r_t cos i) = b1 dx + b2 dy
     float vsys, k, hl, A;
@@ -351,7 +354,9 @@ __device__ __forceinline__ void los_disc2(const DiscConst &d, float x, float y, 
     ta = rsqrt_approx(wa);
     tb = rsqrt_approx(wb);
     const f32x2 t = pk2(ta, tb), u0 = mul2(pk2(wa, wb), t);
-    const f32x2 u = mul2(u0, fma2(mul2(u0, t), dup2(-0.5f), dup2(1.5f)));  // one Newton step
+    const f32x2 nt = fma2(mul2(u0, t), dup2(-0.5f), dup2(1.5f));         // one Newton step
+    const f32x2 u = mul2(u0, nt);
+    upk2(mul2(t, nt), ta, tb);                                           // 1 / u
     upk2(u, ua, ub);
     const float pa = atan_over(fminf(ua, ta)), pb = atan_over(fminf(ub, tb));
     float fa, fb;
