@@ -134,6 +134,8 @@ __device__ void fused_setup(const Geom &g, const FusedSmem &L, int row0, int row
 template <int NT, int MINB, bool RAGGED>
 __global__ void __launch_bounds__(NT, MINB) fused_eval_kernel(FusedArgs a)
 {
+    // a survey's tile classes may start beside this launch (k_tile.cu)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     cg::cluster_group cluster = cg::this_cluster();
     const int cs = a.cs;
     const int rank = (int)cluster.block_rank();

@@ -122,8 +122,7 @@ struct TileDims {
     int PP, RP;      // floats of a plane of a row pair, and of a row pair (padded: see the x pass)
 };
 
-template <int R>
-__device__ __forceinline__ TileDims tile_dims(const Geom &g, int tx, int ty, int tiles_x, int model, int tile)
+__device__ __forceinline__ TileDims tile_dims(const Geom &g, int R, int tx, int ty, int tiles_x, int model, int tile)
 {
     TileDims d;
     d.model = model;
@@ -162,7 +161,7 @@ __device__ __forceinline__ void setup_item(const Geom &g, const TileArgs &a, int
         m.lt = line_table_plan(g, m.mc, m.lc);
     } else if (lane == 1) {
         const int model = it / a.tiles;
-        m.d = tile_dims<R>(g, a.tx, a.ty, a.tiles_x, model, it - model * a.tiles);
+        m.d = tile_dims(g, R, a.tx, a.ty, a.tiles_x, model, it - model * a.tiles);
         m.ob = a.obs_list ? a.obs_list[(a.m0 + model) / a.mpg] : a.obs;
     }
 }
@@ -478,10 +477,9 @@ struct TileTaps {
 
 // A geometry's taps, LSF variance and band-edge tables (fused_line.cuh,
 // edge_tables) with the whole block (over a warp); ends with a barrier.
-template <int R>
-__device__ __forceinline__ void tile_tables(const Geom &g, TileTaps &T, float *edge, int tid, int nthr)
+__device__ __forceinline__ void tile_tables(const Geom &g, int R, TileTaps &T, float *edge, int tid, int nthr)
 {
-    constexpr int W = 2 * R + 1;
+    const int W = 2 * R + 1;
     const int lane = tid & 31, etl = edge_table_len(g);
     for (int j = tid; j <= 2 * g.Rz; j += nthr) T.lz[j] = tap_raw(j - g.Rz, g.sig_z, g.Rz);
     if (tid < W) T.w[tid] = tap_raw(tid - R, g.sig_xy, R);
@@ -500,7 +498,6 @@ __device__ __forceinline__ void tile_tables(const Geom &g, TileTaps &T, float *e
         if (lane == 0) T.var = g.dv * g.dv * (V / S);
         if (lane < W) {
             S = 0.f;
-#pragma unroll
             for (int j = 0; j < W; ++j) S += T.w[j];
             const float w = T.w[lane] / S;
             T.w2[lane] = pk2(w, w);
@@ -563,7 +560,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) tile_kernel(const __grid_cons
     // the geometry's tables: taps, LSF variance, band edges (fused_line.cuh, edge_tables)
     double pv = 1.0;
     if (tid < GBK_NPAR) pv = a.params[(size_t)(it / tiles) * GBK_NPAR + tid];
-    tile_tables<R>(g, T, edge, tid, nthr);
+    tile_tables(g, R, T, edge, tid, nthr);
     if (tid < 32) setup_item<R>(g, a, it, pv, lane, T.var, s_m[0]);
     __syncthreads();
 
@@ -609,7 +606,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) tile_kernel(const __grid_cons
         it = nxt;
         fresh = !same;
         if (same) {
-            if (tid == 0) s_m[buf].d = tile_dims<R>(g, a.tx, a.ty, a.tiles_x, it / tiles, it % tiles);
+            if (tid == 0) s_m[buf].d = tile_dims(g, R, a.tx, a.ty, a.tiles_x, it / tiles, it % tiles);
             __syncthreads();
         } else {
             buf ^= 1;
@@ -619,11 +616,24 @@ __global__ void __launch_bounds__(kTileThreads, 2) tile_kernel(const __grid_cons
 
 // Ragged batches: one galaxy's geometry per item, every image whole in one
 // CTA, the items (costliest first) drawn from a work counter as the CTAs
-// become free.  Launched with the CTA size that its largest galaxy's planes
-// leave room for: 768 threads alone on an SM down to 160 with five on it.
+// become free.  A launch has the CTA size that its largest galaxy's planes
+// leave room for, 768 threads alone on an SM down to 160 with five on it, and
+// galaxies of any PSF radius: launches by radius too were up to 45 in a row.
+// The launches of a call overlap (programmatic dependent launch: the next one
+// may start once this one's CTAs have, and none ends before the one before
+// it has), so that one's last galaxies leave their SMs to the next one's first.
 constexpr int kRaggedThreads = 768;
 
+// Both PSF passes, the moments and residuals; the thread's sum of squares.
 template <int R>
+__device__ __forceinline__ float psf_phases(const TileItem &M, uint32_t taps, float *pl, int nx, size_t np,
+                                            float *maps, float *resid, bool want_obs, int vec, int tid, int nthr)
+{
+    x_phase<R>(M, taps, pl, tid, nthr);
+    __syncthreads();
+    return y_phase<R>(M, taps, pl, nx, np, maps, resid, want_obs, vec, tid, nthr);
+}
+
 __global__ void __launch_bounds__(kRaggedThreads, 1) tile_ragged_kernel(const __grid_constant__ TileRagged a)
 {
     extern __shared__ __align__(16) float sm[];
@@ -632,6 +642,7 @@ __global__ void __launch_bounds__(kRaggedThreads, 1) tile_ragged_kernel(const __
     __shared__ Geom g;
     __shared__ int s_item;
     __shared__ double red[kRaggedThreads / 32];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31;
     const uint32_t taps = (uint32_t)__cvta_generic_to_shared(T.w2);
     const bool want_chi2 = (a.chi2 != nullptr), want_obs = want_chi2 || a.resid;
@@ -646,7 +657,7 @@ __global__ void __launch_bounds__(kRaggedThreads, 1) tile_ragged_kernel(const __
         }
         __syncthreads();
         const int it = s_item;
-        if (it >= a.items) return;
+        if (it >= a.items) break;
         const int gal = a.order[it / a.mpg], sub = it % a.mpg;
         const size_t model = (size_t)gal * a.mpg + sub;
         const size_t np = (size_t)g.nx * g.ny, pix = (size_t)a.pix_off[gal] * a.mpg + (size_t)sub * np;
@@ -654,32 +665,42 @@ __global__ void __launch_bounds__(kRaggedThreads, 1) tile_ragged_kernel(const __
         float *const edge = sm, *const ltab = sm + 3 * etl, *const pl = ltab + kLtMaxSeg * kLtSegF;
         double pv = 1.0;
         if (tid < GBK_NPAR) pv = a.params[model * GBK_NPAR + tid];
-        tile_tables<R>(g, T, edge, tid, nthr);
+        tile_tables(g, g.R, T, edge, tid, nthr);
         if (tid < 32) {
             model_const_warp(pv, g, lane, M.mc);
             if (lane == 0) {
                 M.lc = line_ctx(g, M.mc, T.var);
                 M.lt = line_table_plan(g, M.mc, M.lc);
             } else if (lane == 1) {
-                M.d = tile_dims<R>(g, g.nx, g.ny, 1, 0, 0);
+                M.d = tile_dims(g, g.R, g.nx, g.ny, 1, 0, 0);
                 if (want_obs) M.ob = a.obs_list[gal];
             }
         }
         __syncthreads();
         if (M.lt.nseg > 0) line_table_build(g, M.lc, M.lt, edge, etl, ltab, tid, nthr);
-        lines_phase(g, M, R, edge, ltab, pl, tid, nthr);
-        __syncthreads();
-        x_phase<R>(M, taps, pl, tid, nthr);
+        lines_phase(g, M, g.R, edge, ltab, pl, tid, nthr);
         __syncthreads();
         float *const maps = a.maps ? a.maps + 3 * pix : nullptr, *const resid = a.resid ? a.resid + 2 * pix : nullptr;
         const int vec = g.nx % 2 == 0 && ((uintptr_t)maps % 8) == 0 && ((uintptr_t)resid % 8) == 0;
-        const float v = y_phase<R>(M, taps, pl, g.nx, np, maps, resid, want_obs, vec, tid, nthr);
+        float v;
+        switch (g.R) {  // the block's own
+        case 0: v = psf_phases<0>(M, taps, pl, g.nx, np, maps, resid, want_obs, vec, tid, nthr); break;
+        case 1: v = psf_phases<1>(M, taps, pl, g.nx, np, maps, resid, want_obs, vec, tid, nthr); break;
+        case 2: v = psf_phases<2>(M, taps, pl, g.nx, np, maps, resid, want_obs, vec, tid, nthr); break;
+        case 3: v = psf_phases<3>(M, taps, pl, g.nx, np, maps, resid, want_obs, vec, tid, nthr); break;
+        case 4: v = psf_phases<4>(M, taps, pl, g.nx, np, maps, resid, want_obs, vec, tid, nthr); break;
+        case 5: v = psf_phases<5>(M, taps, pl, g.nx, np, maps, resid, want_obs, vec, tid, nthr); break;
+        case 6: v = psf_phases<6>(M, taps, pl, g.nx, np, maps, resid, want_obs, vec, tid, nthr); break;
+        case 7: v = psf_phases<7>(M, taps, pl, g.nx, np, maps, resid, want_obs, vec, tid, nthr); break;
+        default: v = psf_phases<8>(M, taps, pl, g.nx, np, maps, resid, want_obs, vec, tid, nthr); break;
+        }
         if (want_chi2) {
             const double sum = block_chi2(v, red, tid, nthr);
             if (tid == 0) a.chi2[model] = M.mc.valid ? sum : (double)__int_as_float(0x7fc00000);
         }
         __syncthreads();
     }
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // not before the launch before this one
 }
 
 // ---------------------------------------------------------------------------
@@ -831,34 +852,26 @@ int tile_ragged_threads(const Geom &g, size_t *smem)
     return 0;
 }
 
-template <int R>
-static gbk_status launch_ragged_r(const TileRagged &a, int threads, size_t smem, cudaStream_t st)
+gbk_status launch_tile_ragged(const TileRagged &a, int threads, size_t smem, bool overlap, cudaStream_t st)
 {
     static KernelAttrMemo memo;
-    gbk_status s = ensure_kernel_attrs((const void *)tile_ragged_kernel<R>, smem, false, memo,
+    gbk_status s = ensure_kernel_attrs((const void *)tile_ragged_kernel, smem, false, memo,
                                        "ragged tile evaluator: setting its shared memory");
     if (s) return s;
     const int per_sm = (int)std::min<size_t>(227 * 1024 / (smem + 3072), 800 / threads);
-    tile_ragged_kernel<R><<<std::min(a.items, 152 * std::max(1, per_sm)), threads, smem, st>>>(a);
-    const cudaError_t e = cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)std::min(a.items, 152 * std::max(1, per_sm)), 1, 1);
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = overlap ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, tile_ragged_kernel, a);
     if (e != cudaSuccess) return cuda_fail(e, "ragged tile evaluator launch");
     return GBK_OK;
-}
-
-gbk_status launch_tile_ragged(const TileRagged &a, int R, int threads, size_t smem, cudaStream_t st)
-{
-    switch (R) {
-    case 0: return launch_ragged_r<0>(a, threads, smem, st);
-    case 1: return launch_ragged_r<1>(a, threads, smem, st);
-    case 2: return launch_ragged_r<2>(a, threads, smem, st);
-    case 3: return launch_ragged_r<3>(a, threads, smem, st);
-    case 4: return launch_ragged_r<4>(a, threads, smem, st);
-    case 5: return launch_ragged_r<5>(a, threads, smem, st);
-    case 6: return launch_ragged_r<6>(a, threads, smem, st);
-    case 7: return launch_ragged_r<7>(a, threads, smem, st);
-    case 8: return launch_ragged_r<8>(a, threads, smem, st);
-    default: return fail(GBK_EUNSUPPORTED, "tile evaluator: PSF radius %d > %d", R, kTileMaxR);
-    }
 }
 
 }  // namespace gbk

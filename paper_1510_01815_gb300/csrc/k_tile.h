@@ -40,7 +40,7 @@ gbk_status launch_tile(const Geom &g, const TileShape &ts, int n, const double *
                        float *maps, double *chi2, float *resid, const TileScratch &scratch, const SplitBatch *batch,
                        int m0, cudaStream_t st);
 
-// A ragged batch's galaxies of one PSF radius, every image whole in one CTA.
+// A ragged batch's galaxies, every image whole in one CTA.
 // Models gal * mpg + s (s < mpg) of the galaxies order[0 .. items / mpg);
 // galaxy gal's maps and residuals start at pixel pix_off[gal] * mpg.
 struct TileRagged {
@@ -58,6 +58,8 @@ struct TileRagged {
 };
 // The CTA size that serves the galaxy and its shared memory; 0: not served.
 int tile_ragged_threads(const Geom &g, size_t *smem);
-gbk_status launch_tile_ragged(const TileRagged &a, int R, int threads, size_t smem, cudaStream_t st);
+// `overlap`: the launch before it in the stream is another of the same call,
+// of this kernel or a persistent one of the cluster evaluator.
+gbk_status launch_tile_ragged(const TileRagged &a, int threads, size_t smem, bool overlap, cudaStream_t st);
 
 }  // namespace gbk

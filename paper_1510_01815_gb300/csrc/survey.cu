@@ -3,9 +3,10 @@
 // fitting Bekiaris et al. 2015 motivate in Sec. 1 and Sec. 5.
 //
 // A galaxy whose image fits one CTA goes to the one-kernel evaluator
-// (k_tile.cu): one launch per PSF radius and CTA size, costliest galaxy
-// first from a work counter.  The others, and surveys with a tuning, take the
-// cluster evaluator (k_fused.cu) in one of two ways:
+// (k_tile.cu): one launch per CTA size, costliest galaxy first from a work
+// counter, the launches overlapping.  The others, and every galaxy of a survey
+// with a tuning, take the cluster evaluator (k_fused.cu) in one of two ways,
+// the first unless a tuning says otherwise:
 //  * one persistent launch: a resident wave of thread-block clusters of one
 //    size (the smallest that fits every galaxy two CTAs to an SM) takes the
 //    models, costliest galaxy first, from a work counter as each cluster
@@ -38,8 +39,8 @@ static size_t al256(size_t b) { return (b + 255) & ~(size_t)255; }
 constexpr size_t kSurveySmemCap = 228 * 1024 / 2 - 3 * 1024;
 
 // Work counters at the end of the tables: a persistent cluster launch's two,
-// then one for each tile class (at most five CTA sizes and nine PSF radii).
-constexpr int kSurveyCounters = 64;
+// then one for each tile class (at most five CTA sizes).
+constexpr int kSurveyCounters = 8;
 
 // One persistent launch unless a survey tuning says otherwise.
 constexpr int kSurveyDefaultOne = 1;
@@ -99,12 +100,12 @@ static int one_launch_cs(const std::vector<Geom> &geo, int threads, size_t *smem
     return 0;
 }
 
-// One cluster launch per group of galaxies order[beg .. end) of the same
-// cluster and block size.
-static gbk_status cluster_groups(SurveyPlan *sp, int beg, int end, const std::vector<int> &cs_of,
-                                 const std::vector<int> &thr_of)
+// One cluster launch per group of galaxies (in order) of the same cluster and
+// block size.
+static gbk_status cluster_groups(SurveyPlan *sp, const std::vector<int> &cs_of, const std::vector<int> &thr_of)
 {
-    for (int k = beg; k < end;) {
+    const int end = sp->n_gal;
+    for (int k = 0; k < end;) {
         int i0 = sp->order[k], e = k;
         while (e < end && cs_of[sp->order[e]] == cs_of[i0] && thr_of[sp->order[e]] == thr_of[i0]) ++e;
         SurveyClass c;
@@ -124,49 +125,88 @@ static gbk_status cluster_groups(SurveyPlan *sp, int beg, int end, const std::ve
     return GBK_OK;
 }
 
-// Moves the galaxies that the one-kernel evaluator serves to classes of their
-// own, by CTA size (largest first: the launches run one after the other, and
-// the last one's tail is the short items') and PSF radius; the others stay on
-// the cluster evaluator.  A survey of 2048 galaxies of 24 - 96 spaxels took
-// 546 us on one cluster launch, 243 us on these.
+// One persistent cluster launch over the galaxies `gal` (tu.cs CTAs per
+// cluster; 0: the smallest size that serves them), appended to the plan:
+// first the galaxies that need a cluster, then the ones a single CTA serves;
+// each share costliest first.
 template <class Cost>
-static gbk_status tile_classes(SurveyPlan *sp, const std::vector<int> &cs_of, const std::vector<int> &thr_of,
-                               const Cost &cost)
+static gbk_status one_launch(SurveyPlan *sp, std::vector<int32_t> gal, const SurveyTuning &tu, const Cost &cost)
 {
-    const int n = sp->n_gal;
-    std::vector<int> thr(n);
-    std::vector<size_t> smem(n);
-    int served = 0;
-    for (int i = 0; i < n; ++i) served += (thr[i] = tile_ragged_threads(sp->geo[i], &smem[i])) > 0;
-    if (!served) return GBK_OK;
-    std::stable_sort(sp->order.begin(), sp->order.end(), [&](int a, int b) {
-        if ((thr[a] > 0) != (thr[b] > 0)) return thr[a] == 0;
-        if (thr[a] == 0) {
-            if (cs_of[a] != cs_of[b]) return cs_of[a] > cs_of[b];
-            if (thr_of[a] != thr_of[b]) return thr_of[a] > thr_of[b];
-        } else {
-            if (thr[a] != thr[b]) return thr[a] > thr[b];
-            if (sp->geo[a].R != sp->geo[b].R) return sp->geo[a].R > sp->geo[b].R;
+    SurveyClass c;
+    c.threads = tu.threads;
+    std::vector<char> solo(sp->n_gal);
+    std::vector<Geom> all, big;
+    for (int i : gal) {
+        all.push_back(sp->geo[i]);
+        solo[i] = solo_fits(sp->geo[i], c.threads);
+        if (!solo[i]) big.push_back(sp->geo[i]);
+    }
+    if (tu.cs > 0) {
+        c.cs = tu.cs;
+        if (big.empty()) big = all;  // every galaxy is served by the clusters
+        if (!fused_config_ragged(big.data(), (int)big.size(), c.cs, c.threads, &c.smem))
+            return fail(GBK_EINVAL, "survey tuning: %d-CTA clusters of %d threads do not fit every galaxy", c.cs,
+                        c.threads);
+    } else if (!(c.cs = one_launch_cs(all, c.threads, &c.smem))) {
+        return fail(GBK_EUNSUPPORTED, "no cluster size fits every galaxy of the survey");
+    }
+    // solo galaxies only where a cluster share exists (with none, the
+    // clusters serve everything)
+    const bool split = big.size() < gal.size() && !big.empty() && c.cs > 1;
+    c.n_solo = 0;
+    if (split) {
+        for (int i : gal) {
+            if (!solo[i]) continue;
+            size_t need;
+            fused_config_ragged(&sp->geo[i], 1, 1, c.threads, &need);
+            c.smem = std::max(c.smem, need);
+            ++c.n_solo;
         }
+    } else {
+        std::fill(solo.begin(), solo.end(), 0);
+        if (!fused_config_ragged(all.data(), (int)all.size(), c.cs, c.threads, &c.smem))
+            return fail(GBK_EINVAL, "survey tuning: %d-CTA clusters of %d threads do not fit every galaxy", c.cs,
+                        c.threads);
+    }
+    std::stable_sort(gal.begin(), gal.end(), [&](int a, int b) {
+        if (solo[a] != solo[b]) return solo[a] < solo[b];
+        return cost(a) > cost(b);
+    });
+    c.beg = (int)sp->order.size();
+    c.end = c.beg + (int)gal.size();
+    c.persistent = 1;
+    sp->order.insert(sp->order.end(), gal.begin(), gal.end());
+    sp->classes.push_back(c);
+    return GBK_OK;
+}
+
+// The galaxies that the one-kernel evaluator serves, appended to the plan as
+// classes by CTA size, largest first (the last launch's tail is the short
+// items').  Surveys of 24 - 96 spaxels, cluster launch -> here: 2048 galaxies
+// 563 -> 192 us (PSF radii 3 to 7 mixed: 499 -> 196 us), 256 98 -> 39 us, 16
+// 44 -> 36 us; seven in eight too large for a CTA: 256 338 -> 318 us, 16 53 ->
+// 53 us.
+template <class Cost>
+static void tile_classes(SurveyPlan *sp, std::vector<int32_t> gal, const std::vector<int> &thr,
+                         const std::vector<size_t> &smem, const Cost &cost)
+{
+    std::sort(gal.begin(), gal.end(), [&](int a, int b) {
+        if (thr[a] != thr[b]) return thr[a] > thr[b];
         if (cost(a) != cost(b)) return cost(a) > cost(b);
         return a < b;
     });
-    sp->classes.clear();
-    gbk_status s = cluster_groups(sp, 0, n - served, cs_of, thr_of);
-    if (s) return s;
-    for (int k = n - served; k < n;) {
-        const int i0 = sp->order[k];
+    for (size_t k = 0; k < gal.size();) {
         SurveyClass c = {};
         c.tile = 1;
-        c.R = sp->geo[i0].R;
-        c.threads = thr[i0];
-        c.beg = k;
-        for (; k < n && thr[sp->order[k]] == c.threads && sp->geo[sp->order[k]].R == c.R; ++k)
-            c.smem = std::max(c.smem, smem[sp->order[k]]);
-        c.end = k;
+        c.threads = thr[gal[k]];
+        c.beg = (int)sp->order.size();
+        for (; k < gal.size() && thr[gal[k]] == c.threads; ++k) {
+            c.smem = std::max(c.smem, smem[gal[k]]);
+            sp->order.push_back(gal[k]);
+        }
+        c.end = (int)sp->order.size();
         sp->classes.push_back(c);
     }
-    return GBK_OK;
 }
 
 gbk_status survey_plan(const gbk_geom *geoms, int n_gal, SurveyPlan *sp, const SurveyTuning *force)
@@ -215,72 +255,46 @@ gbk_status survey_plan(const gbk_geom *geoms, int n_gal, SurveyPlan *sp, const S
             tuned = true;
         }
     }
-    sp->order.resize(n_gal);
-    std::iota(sp->order.begin(), sp->order.end(), 0);
+    std::vector<int32_t> all(n_gal);
+    std::iota(all.begin(), all.end(), 0);
+    sp->order.clear();
     sp->classes.clear();
     if (tu.one && n_gal > 0) {
-        // one persistent launch: the galaxies that need a cluster first, then
-        // the ones a single CTA serves; each share costliest first
-        SurveyClass c;
-        c.threads = tu.threads;
-        std::vector<char> solo(n_gal);
-        std::vector<Geom> big;
-        for (int i = 0; i < n_gal; ++i) {
-            solo[i] = solo_fits(sp->geo[i], c.threads);
-            if (!solo[i]) big.push_back(sp->geo[i]);
-        }
-        if (tu.cs > 0) {
-            c.cs = tu.cs;
-            if (big.empty()) big = sp->geo;  // every galaxy is served by the clusters
-            if (!fused_config_ragged(big.data(), (int)big.size(), c.cs, c.threads, &c.smem))
-                return fail(GBK_EINVAL, "survey tuning: %d-CTA clusters of %d threads do not fit every galaxy", c.cs,
-                            c.threads);
-        } else if (!(c.cs = one_launch_cs(sp->geo, c.threads, &c.smem))) {
-            return fail(GBK_EUNSUPPORTED, "no cluster size fits every galaxy of the survey");
-        }
-        // solo galaxies only where a cluster share exists (with none, the
-        // clusters serve everything)
-        const bool split = (int)big.size() < n_gal && !big.empty() && c.cs > 1;
-        c.n_solo = 0;
-        if (split) {
-            for (int i = 0; i < n_gal; ++i) {
-                if (!solo[i]) continue;
-                size_t need;
-                fused_config_ragged(&sp->geo[i], 1, 1, c.threads, &need);
-                c.smem = std::max(c.smem, need);
-                ++c.n_solo;
-            }
-        } else {
-            std::fill(solo.begin(), solo.end(), 0);
-            if (!fused_config_ragged(sp->geo.data(), n_gal, c.cs, c.threads, &c.smem))
-                return fail(GBK_EINVAL, "survey tuning: %d-CTA clusters of %d threads do not fit every galaxy", c.cs,
-                            c.threads);
-        }
-        c.beg = 0;
-        c.end = n_gal;
-        c.persistent = 1;
-        std::stable_sort(sp->order.begin(), sp->order.end(), [&](int a, int b) {
-            if (solo[a] != solo[b]) return solo[a] < solo[b];
-            return cost(a) > cost(b);
-        });
-        sp->classes.push_back(c);
-        tu.cs = c.cs;
+        gbk_status s = one_launch(sp, all, tu, cost);
+        if (s) return s;
+        tu.cs = sp->classes[0].cs;
     }
-    // groups: larger clusters first, then costliest first; ties by index
-    if (!tu.one)
+    if (!tu.one) {
+        // groups: larger clusters first, then costliest first; ties by index
+        sp->order = all;
         std::stable_sort(sp->order.begin(), sp->order.end(), [&](int a, int b) {
             if (cs_of[a] != cs_of[b]) return cs_of[a] > cs_of[b];
             if (thr_of[a] != thr_of[b]) return thr_of[a] > thr_of[b];
             return cost(a) > cost(b);
         });
-    sp->tuning = tu;
-    if (!tu.one) {
-        gbk_status s = cluster_groups(sp, 0, n_gal, cs_of, thr_of);
+        gbk_status s = cluster_groups(sp, cs_of, thr_of);
         if (s) return s;
     }
+    sp->tuning = tu;
     if (!tuned) {
-        gbk_status s = tile_classes(sp, cs_of, thr_of, cost);
-        if (s) return s;
+        // the one-kernel evaluator where it serves a galaxy, the persistent
+        // launch for the others
+        std::vector<int> thr(n_gal);
+        std::vector<size_t> smem(n_gal);
+        std::vector<int32_t> served, rest;
+        for (int i = 0; i < n_gal; ++i) {
+            thr[i] = tile_ragged_threads(sp->geo[i], &smem[i]);
+            (thr[i] > 0 ? served : rest).push_back(i);
+        }
+        if (!served.empty()) {
+            sp->order.clear();
+            sp->classes.clear();
+            if (!rest.empty()) {
+                gbk_status s = one_launch(sp, rest, SurveyTuning{1, 0, tu.threads}, cost);
+                if (s) return s;
+            }
+            tile_classes(sp, served, thr, smem, cost);
+        }
     }
     // classes of the analytic Jacobian kernel: smallest cluster whose CTAs fit
     std::vector<int> tcs(n_gal);
@@ -469,7 +483,9 @@ gbk_status survey_eval(const SurveyPlan &sp, int mpg, const double *params, cons
         if (c.tile) {
             const TileRagged t = {sp.d_geo, sp.d_pix_off, d_order + c.beg, params, obs_list, skip, maps, chi2, resid,
                                   work++,   (c.end - c.beg) * mpg,          mpg};
-            gbk_status s = launch_tile_ragged(t, c.R, c.threads, c.smem, st);
+            // (a persistent launch lets the next one start, as a tile class does)
+            const bool overlap = ci > 0 && (classes[ci - 1].tile || classes[ci - 1].persistent);
+            gbk_status s = launch_tile_ragged(t, c.threads, c.smem, overlap, st);
             if (s) return s;
             continue;
         }

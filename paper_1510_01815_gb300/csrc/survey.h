@@ -16,8 +16,7 @@ struct SurveyClass {
     int persistent;  // 1: one resident wave of clusters fed by the work counters
     int n_solo;      // persistent: the last n_solo galaxies of the range go to single CTAs
     int direct = 0;  // Jacobian classes: halo rows read in the neighbours' shared memory
-    int tile = 0;    // 1: images whole in one CTA (k_tile.cu) of `threads` threads, PSF radius R
-    int R = 0;
+    int tile = 0;    // 1: images whole in one CTA (k_tile.cu) of `threads` threads
 };
 
 // How the fused evaluator serves a survey: one launch per class (one = 0),
