@@ -346,20 +346,24 @@ def run_survey(gbk, torch, n, n_plain, device):
         b.synchronize()
         return a.elapsed_time(b) / reps
 
-    # launch shapes: one launch per cluster-size group, the default single
-    # persistent launch, and the autotuner's choice (kept for the fits below)
+    # launch shapes: one cluster launch per cluster-size group, one persistent
+    # cluster launch, the default, and the autotuner's choice (kept for the
+    # fits below)
     shapes = {}
     gbk.gbk_survey_set_tuning(geoms, 0)
     shapes["per_group_launches"] = time_eval()
     gbk.gbk_survey_set_tuning(geoms, None)
-    t_def = gbk.gbk_survey_get_tuning(geoms)
-    shapes["one_launch_%dx%d" % (t_def["cluster_ctas"], t_def["threads"])] = time_eval()
+    shapes["default_one_kernel"] = time_eval()
+    cs = gbk.gbk_survey_get_tuning(geoms)["cluster_ctas"]
+    gbk.gbk_survey_set_tuning(geoms, 1, cs, 512)
+    shapes["one_launch_%dx512" % cs] = time_eval()
     best = gbk.gbk_survey_autotune(geoms, d_p, obs_dev, d_c, ws)
     ms = time_eval()
     out["eval"] = {"ms_per_survey": ms, "evals_per_s": n / (ms * 1e-3), "data_voxels_per_s": vox / (ms * 1e-3),
                    "tuning": best, "shapes_ms": shapes,
-                   "note": "time per call: cached plan, geometry-table upload, counter reset and the fused "
-                           "launch(es); tuning = the survey autotuner's choice, used by the fits below"}
+                   "note": "time per call: cached plan, geometry-table upload, counter reset and the "
+                           "launch(es) of the survey autotuner's choice, used by the fits below (the "
+                           "default's cluster shape where the default was the fastest)"}
     for name, mode, jac, sub, path in (("batched_tangent", gbk.LM_BATCHED, gbk.JAC_TANGENT, n, gbk.PATH_AUTO),
                                        ("batched_tangent_cluster_kernels", gbk.LM_BATCHED, gbk.JAC_TANGENT, n,
                                         gbk.PATH_FUSED),

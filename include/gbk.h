@@ -571,12 +571,17 @@ GBK_API gbk_status gbk_nested_sample_traced(const gbk_geom *g, const gbk_obs *ob
                                             double *post_std, double *log_z, int64_t *n_eval, int32_t *n_iter,
                                             void *workspace, size_t ws_bytes, void *stream, gbk_ns_trace *trace);
 
-/* Launch tuning of the fused path (no counterpart in the paper).  A tuning
- * is the number of CTAs that cooperate on one model (a thread-block cluster
- * of 1..16 CTAs sharing the model's extended rows through distributed shared
- * memory), the block size (512, 384 or 256 threads) and the grid shape.  The library keeps
- * one tuning per geometry (size, kernel radii, LSF mode) for the life of the
- * process; without one it uses a heuristic. */
+/* Launch tuning of the fused path (no counterpart in the paper).  Without a
+ * tuning a fused call takes the one-kernel evaluator (a CTA per image or tile)
+ * where that needs no workspace: the cube model with PSF radii up to 8 px,
+ * maps of any image and chi2 of images that fit one CTA.  Other calls take the
+ * cluster kernel in a heuristic shape.  A tuning is a shape of the cluster
+ * kernel -- the number of CTAs that cooperate on one model (a thread-block
+ * cluster of 1..16 CTAs sharing the model's extended rows through distributed
+ * shared memory), the block size (512, 384 or 256 threads) and the grid
+ * shape -- and one that a caller sets also keeps the calls on that kernel which
+ * the one-kernel evaluator would serve.  The library keeps one tuning per
+ * geometry (size, kernel radii, LSF mode) for the life of the process. */
 typedef struct gbk_tuning {
     int32_t cluster_ctas;  /* CTAs per model                                  */
     int32_t threads;       /* threads per CTA                                 */
@@ -587,34 +592,45 @@ typedef struct gbk_tuning {
 } gbk_tuning;
 
 /* Times every valid tuning of the fused path on this batch (params, obs and
- * chi2_scratch as for gbk_chi2; chi2_scratch is overwritten) and keeps the
- * fastest for this geometry.  Synchronises `stream`; several launches per
+ * chi2_scratch as for gbk_chi2; chi2_scratch is overwritten), the one-kernel
+ * evaluator among them where it serves the batch, and keeps the fastest for
+ * this geometry: where the one-kernel evaluator is, the geometry has no tuning
+ * afterwards and best is what gbk_get_tuning reports without one (there is no
+ * tuning to save then).  Synchronises `stream`; several launches per
  * candidate.  best (host) receives the choice.  Call it outside any stream
  * capture. */
 GBK_API gbk_status gbk_autotune(const gbk_geom *g, int32_t n_models, const double *params,
                                 const gbk_obs *obs, double *chi2_scratch, gbk_tuning *best,
                                 void *stream);
 
-/* The tuning the next fused call with this geometry will use (host out). */
+/* The cluster kernel's shape for this geometry (host out): the tuning, or
+ * without one the heuristic shape, which calls that the one-kernel evaluator
+ * serves do not use. */
 GBK_API gbk_status gbk_get_tuning(const gbk_geom *g, gbk_tuning *out);
 
 /* Sets the tuning for this geometry (e.g. one saved from an earlier
- * gbk_autotune); t == NULL forgets it.  EINVAL if it cannot run here. */
+ * gbk_autotune) and keeps its fused calls on the cluster kernel; t == NULL
+ * forgets it.  EINVAL if it cannot run here. */
 GBK_API gbk_status gbk_set_tuning(const gbk_geom *g, const gbk_tuning *t);
 
-/* Survey tunings: how the fused evaluator serves one survey (keyed by the
- * sizes, kernel radii and LSF modes of its geometry list).  persistent = 1:
- * one persistent launch of cluster_ctas-CTA clusters of `threads` threads
- * over every galaxy; persistent = 0: one launch per cluster-size group
- * (cluster_ctas and threads 0).  gbk_survey_autotune times the per-group
- * launches and one launch with 512 and 256 threads at the four smallest
- * cluster sizes that fit every galaxy, on gbk_survey_eval of `params`
- * against `obs` (chi2_scratch [n_gal] is overwritten; the workspace is that
- * of gbk_survey_workspace_bytes(geoms, n_gal, NULL)), keeps the fastest for
- * this survey and returns it in best (host).  Synchronises `stream`; call
- * it outside any stream capture.  gbk_survey_get_tuning reports the shape
- * the next survey call will use; gbk_survey_set_tuning sets one (EINVAL if
- * it does not fit every galaxy) or, with t == NULL, forgets it. */
+/* Survey tunings (keyed by the sizes, kernel radii and LSF modes of the
+ * geometry list).  Without one, galaxies that fit one CTA take the one-kernel
+ * evaluator (one launch per CTA size, overlapping) and the others a persistent
+ * cluster launch; a tuning puts every galaxy on the cluster evaluator.
+ * persistent = 1: one persistent launch of cluster_ctas-CTA clusters of
+ * `threads` threads over every galaxy; persistent = 0: one launch per
+ * cluster-size group (cluster_ctas and threads 0).  gbk_survey_autotune times
+ * the untuned launches, the per-group launches and one launch with 512 and 256
+ * threads at the four smallest cluster sizes that fit every galaxy, on
+ * gbk_survey_eval of `params` against `obs` (chi2_scratch [n_gal] is
+ * overwritten; the workspace is that of gbk_survey_workspace_bytes(geoms,
+ * n_gal, NULL)), keeps the fastest for this survey and returns it in best
+ * (host); where the untuned launches are the fastest the survey has no tuning
+ * afterwards and best is what gbk_survey_get_tuning reports without one.
+ * Synchronises `stream`; call it outside any stream capture.
+ * gbk_survey_get_tuning reports the tuning, or without one the cluster shape
+ * that would serve every galaxy; gbk_survey_set_tuning sets one (EINVAL if it
+ * does not fit every galaxy) or, with t == NULL, forgets it. */
 GBK_API gbk_status gbk_survey_autotune(const gbk_geom *geoms, int32_t n_gal, const double *params,
                                        const gbk_obs *obs, double *chi2_scratch, void *workspace, size_t ws_bytes,
                                        gbk_tuning *best, void *stream);

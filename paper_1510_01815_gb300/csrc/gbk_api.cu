@@ -267,18 +267,30 @@ static gbk_status run_staged(const Geom &g, int32_t n, const double *params, flo
     return ok();
 }
 
-static gbk_status run_fused(const Geom &g, int32_t n, const double *params, float *maps, const gbk_obs *obs,
-                            double *chi2, float *resid, cudaStream_t st)
+}  // extern "C"
+
+namespace gbk {
+
+bool fused_tile_shape(const Geom &g, int32_t n, bool chi2, TileShape *ts)
 {
+    return g.ex <= 1024 && tile_shape(g, chi2 ? kTileChi2Batch : n, chi2, ts) && n <= 0x7fffffff / ts->tiles;
+}
+
+gbk_status run_fused(const Geom &g, int32_t n, const double *params, float *maps, const gbk_obs *obs, double *chi2,
+                     float *resid, const FusedConfig *fc, cudaStream_t st)
+{
+    if (n == 0) return GBK_OK;
+    if (!fc) {
+        TileShape ts;
+        if (!fused_tile_shape(g, n, chi2 != nullptr, &ts))
+            return fail(GBK_EUNSUPPORTED, "the one-kernel evaluator does not serve this call");
+        return launch_tile(g, ts, n, params, obs, maps, chi2, resid, TileScratch(), nullptr, 0, st);
+    }
     FusedArgs a = {};
-    FusedConfig fc;
-    if (!fused_config(g, &fc))
-        return fail(GBK_EUNSUPPORTED, "the fused path cannot serve this geometry (upsample %d, %d x %d)", g.u,
-                    g.nx, g.ny);
-    a.cs = fc.cs;
-    a.band = fc.band;
-    a.threads = fc.threads;
-    a.persistent = fc.persistent;
+    a.cs = fc->cs;
+    a.band = fc->band;
+    a.threads = fc->threads;
+    a.persistent = fc->persistent;
     a.g = g;
     a.n_models = n;
     a.params = params;
@@ -286,22 +298,31 @@ static gbk_status run_fused(const Geom &g, int32_t n, const double *params, floa
     a.maps = maps;
     a.chi2 = chi2;
     a.resid = resid;
-    if (n == 0) return ok();
-    // The one-kernel evaluator where it needs no workspace either: without
-    // chi2 any image, with it an image that fits one CTA (its chi2 parts have
-    // nowhere to meet).  A call for the maps of 77 models of 57 x 43 x 37,
-    // alone: 58 us on the cluster kernel, 43 us on this one.  A geometry whose
-    // cluster launch was tuned keeps it.
+    return launch_fused(a, st);
+}
+
+}  // namespace gbk
+
+// The fused path: the one-kernel evaluator where it needs no workspace either
+// -- without chi2 any image, with it an image that fits one CTA (its chi2 parts
+// have nowhere to meet) -- else the cluster kernel.  Maps of 64 models of 128 x
+// 128 x 64: 69 us on the cluster kernel, 33 us on this one.  A tuning that pins
+// the cluster kernel for the geometry keeps it there.
+static gbk_status call_fused(const Geom &g, int32_t n, const double *params, float *maps, const gbk_obs *obs,
+                             double *chi2, float *resid, cudaStream_t st)
+{
+    FusedConfig fc;
+    if (!fused_config(g, &fc))
+        return fail(GBK_EUNSUPPORTED, "the fused path cannot serve this geometry (upsample %d, %d x %d)", g.u,
+                    g.nx, g.ny);
     TileShape ts;
-    gbk_status s;
-    if (g.ex <= 1024 && !fused_tuned(g) && tile_shape(g, chi2 ? kTileChi2Batch : n, chi2 != nullptr, &ts) &&
-        n <= 0x7fffffff / ts.tiles)
-        s = launch_tile(g, ts, n, params, obs, maps, chi2, resid, TileScratch(), nullptr, 0, st);
-    else
-        s = launch_fused(a, st);
+    const bool tile = !fused_pinned(g) && fused_tile_shape(g, n, chi2 != nullptr, &ts);
+    gbk_status s = run_fused(g, n, params, maps, obs, chi2, resid, tile ? nullptr : &fc, st);
     if (s) return s;
     return ok();
 }
+
+extern "C" {
 
 gbk_status gbk_eval_cubes(const gbk_geom *gin, int32_t n_models, const double *params, float *cubes,
                           float *maps, void *workspace, size_t ws_bytes, void *stream)
@@ -325,7 +346,7 @@ gbk_status gbk_eval_cubes(const gbk_geom *gin, int32_t n_models, const double *p
     }
     if (cubes || !fused_config(g, &fc))
         return run_staged(g, n_models, params, cubes, maps, nullptr, nullptr, nullptr, workspace, ws_bytes, st);
-    return run_fused(g, n_models, params, maps, nullptr, nullptr, nullptr, st);
+    return call_fused(g, n_models, params, maps, nullptr, nullptr, nullptr, st);
 }
 
 gbk_status gbk_chi2(const gbk_geom *gin, int32_t n_models, const double *params, const gbk_obs *obs,
@@ -351,7 +372,7 @@ gbk_status gbk_chi2(const gbk_geom *gin, int32_t n_models, const double *params,
     }
     if (flags == GBK_PATH_STAGED || (flags == GBK_PATH_AUTO && !fused_ok))
         return run_staged(g, n_models, params, nullptr, nullptr, obs, chi2, resid, workspace, ws_bytes, st);
-    return run_fused(g, n_models, params, nullptr, obs, chi2, resid, st);
+    return call_fused(g, n_models, params, nullptr, obs, chi2, resid, st);
 }
 
 // Workspace of gbk_chi2_host: the device copies of the parameters, the

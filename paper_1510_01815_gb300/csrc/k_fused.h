@@ -57,10 +57,18 @@ struct FusedConfig {
 size_t fused_smem_bytes_host(const Geom &g, int band);
 bool fused_config_ragged(const Geom *geoms, int n, int cs, int threads, size_t *smem);
 bool fused_config(const Geom &g, FusedConfig *cfg);
-// A tuning was set for this geometry (by the caller or the autotuner).
-bool fused_tuned(const Geom &g);
+// A tuning keeps this geometry on the cluster kernel also where the one-kernel
+// evaluator serves the call.
+bool fused_pinned(const Geom &g);
 bool fused_config_valid(const Geom &g, int cs, int threads, int persistent, FusedConfig *cfg);
 gbk_status launch_fused(const FusedArgs &args, cudaStream_t stream);
+// Maps, chi2 or residuals by the cluster kernel in the shape *fc, or (fc null)
+// by the one-kernel evaluator without a workspace, which serves the call where
+// fused_tile_shape finds a shape (gbk_api.cu).
+struct TileShape;
+bool fused_tile_shape(const Geom &g, int32_t n, bool chi2, TileShape *ts);
+gbk_status run_fused(const Geom &g, int32_t n, const double *params, float *maps, const gbk_obs *obs, double *chi2,
+                     float *resid, const FusedConfig *fc, cudaStream_t st);
 // Velocity-field models (k_vfield.cu); launch_fused dispatches to it.
 gbk_status launch_vfield(const FusedArgs &args, cudaStream_t stream);
 

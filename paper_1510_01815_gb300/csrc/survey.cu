@@ -13,8 +13,8 @@
 //    becomes free;
 //  * one launch per class: the galaxies grouped by the smallest cluster that
 //    fits each of them, one cluster per model, each group costliest first.
-// A per-survey autotuner (gbk_survey_autotune) times both shapes and caches
-// the winner for the survey's geometry list.  The geometry table, the packed
+// A per-survey autotuner (gbk_survey_autotune) times the default and both
+// shapes and caches the winner for the survey's geometry list.  The geometry table, the packed
 // pixel offsets, the orders and the work counter live at the start of the
 // caller's workspace.
 #include <algorithm>
@@ -209,7 +209,7 @@ static void tile_classes(SurveyPlan *sp, std::vector<int32_t> gal, const std::ve
     }
 }
 
-gbk_status survey_plan(const gbk_geom *geoms, int n_gal, SurveyPlan *sp, const SurveyTuning *force)
+gbk_status survey_plan(const gbk_geom *geoms, int n_gal, SurveyPlan *sp, const SurveyTuning *force, bool untuned)
 {
     if (!geoms) return fail(GBK_EINVAL, "geoms is NULL");
     if (n_gal < 0) return fail(GBK_EINVAL, "n_gal must be >= 0");
@@ -247,7 +247,7 @@ gbk_status survey_plan(const gbk_geom *geoms, int n_gal, SurveyPlan *sp, const S
     bool tuned = force != nullptr;
     if (force) {
         tu = *force;
-    } else if (n_gal > 0) {
+    } else if (n_gal > 0 && !untuned) {
         std::lock_guard<std::mutex> lk(g_stune_mu);
         auto it = g_stune.find(survey_key(sp->geo));
         if (it != g_stune.end()) {
@@ -661,9 +661,11 @@ gbk_status gbk_survey_autotune(const gbk_geom *geoms, int32_t n_gal, const doubl
         return fail(GBK_EWORKSPACE, "gbk_survey_autotune needs %zu bytes of workspace (got %zu)", base.table_bytes,
                     ws_bytes);
     if ((s = check_device_ptr(workspace, "workspace", 256))) return s;
-    // candidates: the per-class launches, and one launch with 256 or 512
-    // threads and the four smallest cluster sizes that fit every galaxy
-    std::vector<SurveyTuning> cand = {{0, 0, 0}};
+    // candidates: the default (untuned) launches, the per-class launches, and
+    // one launch with 256 or 512 threads and the four smallest cluster sizes
+    // that fit every galaxy
+    const SurveyTuning kDefault = {-1, 0, 0};
+    std::vector<SurveyTuning> cand = {kDefault, {0, 0, 0}};
     for (int threads : {512, 256}) {
         size_t smem;
         const int cs0 = one_launch_cs(base.geo, threads, &smem);
@@ -675,11 +677,13 @@ gbk_status gbk_survey_autotune(const gbk_geom *geoms, int32_t n_gal, const doubl
     cudaEventCreate(&t0);
     cudaEventCreate(&t1);
     SurveyTuning bt = {0, 0, 0};
+    bool keep_default = false;
     float best_ms = 0.f;
     int tried = 0;
     for (const SurveyTuning &c : cand) {
         SurveyPlan p;
-        if (survey_plan(geoms, n_gal, &p, &c) || survey_upload(&p, (char *)workspace, st)) continue;
+        const bool def = c.one < 0;
+        if (survey_plan(geoms, n_gal, &p, def ? nullptr : &c, def) || survey_upload(&p, (char *)workspace, st)) continue;
         if (survey_eval(p, 1, params, obs, nullptr, nullptr, chi2_scratch, nullptr, st)) {  // warm-up
             cudaGetLastError();
             continue;
@@ -702,6 +706,7 @@ gbk_status gbk_survey_autotune(const gbk_geom *geoms, int32_t n_gal, const doubl
         if (tried++ == 0 || med < best_ms) {
             best_ms = med;
             bt = p.tuning;
+            keep_default = def;
         }
     }
     cudaEventDestroy(t0);
@@ -711,7 +716,10 @@ gbk_status gbk_survey_autotune(const gbk_geom *geoms, int32_t n_gal, const doubl
     if (tried == 0) return fail(GBK_EUNSUPPORTED, "no survey launch shape could run");
     {
         std::lock_guard<std::mutex> lk(g_stune_mu);
-        g_stune[survey_key(base.geo)] = bt;
+        if (keep_default)
+            g_stune.erase(survey_key(base.geo));
+        else
+            g_stune[survey_key(base.geo)] = bt;
         ++g_tune_gen;
     }
     best->cluster_ctas = bt.one ? bt.cs : 0;

@@ -48,8 +48,10 @@ struct SurveyPlan {
     int64_t total_pix() const { return pix_off.empty() ? 0 : pix_off.back(); }
 };
 
-// `force` (optional) overrides the cached or default survey tuning.
-gbk_status survey_plan(const gbk_geom *geoms, int n_gal, SurveyPlan *sp, const SurveyTuning *force = nullptr);
+// `force` (optional) overrides the cached or default survey tuning; `untuned`
+// ignores the cached one.
+gbk_status survey_plan(const gbk_geom *geoms, int n_gal, SurveyPlan *sp, const SurveyTuning *force = nullptr,
+                       bool untuned = false);
 // survey_plan through a small cache of recent plans (same geometry bytes,
 // same survey tunings): repeated calls over one survey skip the planning.
 gbk_status survey_plan_cached(const gbk_geom *geoms, int n_gal, SurveyPlan *sp);

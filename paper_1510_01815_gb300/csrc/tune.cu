@@ -1,12 +1,13 @@
-// tune.cu -- launch configuration of the fused kernel: a heuristic default
-// and a measuring autotuner with a per-geometry cache.
+// tune.cu -- launch configuration of the fused path: a heuristic default and a
+// measuring autotuner with a per-geometry cache.
 //
-// A configuration is (cluster size = CTAs per model, block size, grid shape).  The
-// cluster size sets how many extended rows each CTA owns (its shared memory
-// and the balance of the line-sampling work); the block size sets the
-// register budget and the warps per SM.  The autotuner times every valid
-// candidate on the caller's own batch and keeps the fastest for that
-// geometry; later calls with the same geometry use it.
+// A configuration of the cluster kernel is (cluster size = CTAs per model,
+// block size, grid shape).  The cluster size sets how many extended rows each
+// CTA owns (its shared memory and the balance of the line-sampling work); the
+// block size sets the register budget and the warps per SM.  The autotuner
+// times every valid candidate on the caller's own batch, the one-kernel
+// evaluator among them where it serves the call, and keeps the fastest for
+// that geometry; later calls with the same geometry use it.
 #include <algorithm>
 #include <cmath>
 #include <map>
@@ -17,13 +18,21 @@
 
 #include "gbk_api_internal.h"
 #include "k_fused.h"
+#include "k_tile.h"
 
 namespace gbk {
 
 using TuneKey = std::tuple<int, int, int, int, int, int>;
 
+// A geometry's tuning: the cluster kernel's shape and, `pinned`, that it also
+// takes the calls that the one-kernel evaluator would serve.
+struct Tuning {
+    FusedConfig shape;
+    bool pinned;
+};
+
 static std::mutex g_tune_mu;
-static std::map<TuneKey, FusedConfig> g_tune_cache;
+static std::map<TuneKey, Tuning> g_tune_cache;
 
 static TuneKey key_of(const Geom &g) { return TuneKey(g.nx, g.ny, g.nz, g.R, g.Rz, g.lsf_mode); }
 
@@ -90,10 +99,11 @@ static bool heuristic(const Geom &g, FusedConfig *cfg)
     return best > 0.0;
 }
 
-bool fused_tuned(const Geom &g)
+bool fused_pinned(const Geom &g)
 {
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    return g_tune_cache.find(key_of(g)) != g_tune_cache.end();
+    auto it = g_tune_cache.find(key_of(g));
+    return it != g_tune_cache.end() && it->second.pinned;
 }
 
 bool fused_config(const Geom &g, FusedConfig *cfg)
@@ -104,7 +114,7 @@ bool fused_config(const Geom &g, FusedConfig *cfg)
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tune_cache.find(key_of(g));
         if (it != g_tune_cache.end()) {
-            *cfg = it->second;
+            *cfg = it->second.shape;
             return true;
         }
     }
@@ -133,51 +143,47 @@ gbk_status gbk_autotune(const gbk_geom *gin, int32_t n_models, const double *par
     cudaEvent_t t0, t1;
     cudaEventCreate(&t0);
     cudaEventCreate(&t1);
+    // candidates: the one-kernel evaluator (a shape of 0 CTAs) where it serves
+    // the call, then every valid shape of the cluster kernel
+    TileShape ts;
+    const bool tile = fused_tile_shape(g, n_models, true, &ts);
+    std::vector<FusedConfig> cand;
+    if (tile) cand.push_back(FusedConfig{0, 0, 0, 0});
+    for (int pers = 0; pers < 2; ++pers)
+        for (int threads : kBlockSizes)
+            for (int cs = 1; cs <= kFusedMaxCluster; ++cs) {
+                FusedConfig c;
+                if (fused_config_valid(g, cs, threads, pers, &c)) cand.push_back(c);
+            }
+    auto run = [&](const FusedConfig &c) {
+        return run_fused(g, n_models, params, nullptr, obs, chi2_scratch, nullptr, c.cs ? &c : nullptr, st) == GBK_OK;
+    };
+    auto timed = [&](const FusedConfig &c, float *ms) {
+        cudaEventRecord(t0, st);
+        const bool ok_run = run(c);
+        cudaEventRecord(t1, st);
+        cudaEventSynchronize(t1);
+        cudaEventElapsedTime(ms, t0, t1);
+        return ok_run;
+    };
     FusedConfig bestc = {0, 0, 0, 0};
     float best_ms = 0.f;
     int tried = 0;
     std::vector<std::pair<float, FusedConfig>> finalists;  // (screen median, configuration)
-    for (int pers = 0; pers < 2; ++pers) {
-    for (int ti = 0; ti < 3; ++ti) {
-        for (int cs = 1; cs <= kFusedMaxCluster; ++cs) {
-            FusedConfig c;
-            if (!fused_config_valid(g, cs, kBlockSizes[ti], pers, &c)) continue;
-            FusedArgs a = {};
-            a.g = g;
-            a.n_models = n_models;
-            a.params = params;
-            a.obs = *obs;
-            a.chi2 = chi2_scratch;
-            a.cs = c.cs;
-            a.band = c.band;
-            a.threads = c.threads;
-            a.persistent = c.persistent;
-            if (launch_fused(a, st) != GBK_OK) {  // e.g. a cluster shape the device cannot place
-                cudaGetLastError();
-                continue;
-            }
-            float times[3];
-            bool ok_run = true;
-            for (int rep = 0; rep < 3 && ok_run; ++rep) {
-                cudaEventRecord(t0, st);
-                ok_run = launch_fused(a, st) == GBK_OK;
-                cudaEventRecord(t1, st);
-                cudaEventSynchronize(t1);
-                cudaEventElapsedTime(&times[rep], t0, t1);
-            }
-            if (!ok_run) {
-                cudaGetLastError();
-                continue;
-            }
-            float med = std::fmax(std::fmin(times[0], times[1]), std::fmin(std::fmax(times[0], times[1]), times[2]));
-            ++tried;
-            finalists.push_back({med, c});
-            if (bestc.cs == 0 || med < best_ms) {
-                best_ms = med;
-                bestc = c;
-            }
+    for (const FusedConfig &c : cand) {
+        float times[3];
+        bool ok_run = run(c);  // warm-up; fails e.g. for a cluster shape the device cannot place
+        for (int rep = 0; rep < 3 && ok_run; ++rep) ok_run = timed(c, &times[rep]);
+        if (!ok_run) {
+            cudaGetLastError();
+            continue;
         }
-    }
+        float med = std::fmax(std::fmin(times[0], times[1]), std::fmin(std::fmax(times[0], times[1]), times[2]));
+        finalists.push_back({med, c});
+        if (tried++ == 0 || med < best_ms) {
+            best_ms = med;
+            bestc = c;
+        }
     }
     // The screen above takes a median of 3; its four fastest candidates,
     // often within a few per cent of each other, are re-timed with 9
@@ -192,24 +198,8 @@ gbk_status gbk_autotune(const gbk_geom *gin, int32_t n_models, const double *par
         std::vector<std::vector<float>> reps(finalists.size());
         for (int rep = 0; rep < 9; ++rep) {
             for (size_t i = 0; i < finalists.size(); ++i) {
-                const FusedConfig &c = finalists[i].second;
-                FusedArgs a = {};
-                a.g = g;
-                a.n_models = n_models;
-                a.params = params;
-                a.obs = *obs;
-                a.chi2 = chi2_scratch;
-                a.cs = c.cs;
-                a.band = c.band;
-                a.threads = c.threads;
-                a.persistent = c.persistent;
                 float ms = 0.f;
-                cudaEventRecord(t0, st);
-                const bool ok_run = launch_fused(a, st) == GBK_OK;
-                cudaEventRecord(t1, st);
-                cudaEventSynchronize(t1);
-                cudaEventElapsedTime(&ms, t0, t1);
-                if (ok_run) reps[i].push_back(ms);
+                if (timed(finalists[i].second, &ms)) reps[i].push_back(ms);
             }
         }
         for (size_t i = 0; i < finalists.size(); ++i) {
@@ -229,8 +219,12 @@ gbk_status gbk_autotune(const gbk_geom *gin, int32_t n_models, const double *par
     if (tried == 0) return fail(GBK_EUNSUPPORTED, "no fused configuration could run for this geometry");
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
-        g_tune_cache[key_of(g)] = bestc;
+        if (bestc.cs == 0)
+            g_tune_cache.erase(key_of(g));
+        else
+            g_tune_cache[key_of(g)] = Tuning{bestc, tile};
     }
+    if (bestc.cs == 0) fused_config(g, &bestc);  // reported: the default shape
     best->cluster_ctas = bestc.cs;
     best->threads = bestc.threads;
     best->persistent = bestc.persistent;
@@ -269,7 +263,7 @@ gbk_status gbk_set_tuning(const gbk_geom *gin, const gbk_tuning *t)
     if (!fused_config_valid(g, t->cluster_ctas, t->threads, t->persistent, &c))
         return fail(GBK_EINVAL, "cluster_ctas %d / threads %d / persistent %d is not a valid fused configuration here",
                     t->cluster_ctas, t->threads, t->persistent);
-    g_tune_cache[key_of(g)] = c;
+    g_tune_cache[key_of(g)] = Tuning{c, true};
     return ok();
 }
 

@@ -250,8 +250,8 @@ def gbk_chi2(geom, params, obs, chi2, resid=None, flags=PATH_AUTO, workspace=Non
 
 
 def gbk_split_stage_times(geom, params, obs, chi2, workspace, stream=None):
-    """gbk_chi2 on the split path, timed per stage; returns ([set-up, line
-    stage, PSF/moments stage] milliseconds, kernel launches)."""
+    """gbk_chi2 on the split path, timed; returns ([clearing the arrival
+    counters, evaluator, 0] milliseconds, kernel launches)."""
     g = cgeom(geom)
     n = params.shape[0] if params.dim() == 2 else params.numel() // NPAR
     ws_bytes = workspace.numel() * workspace.element_size() if workspace is not None else 0
@@ -323,8 +323,9 @@ def gbk_measure_alu_peak(stream=None):
 
 
 def gbk_autotune(geom, params, obs, chi2_scratch, stream=None):
-    """Times the fused-path tunings on this batch and keeps the fastest for
-    the geometry; returns a dict of the choice."""
+    """Times the fused-path tunings and the one-kernel evaluator on this batch
+    and keeps the fastest for the geometry (no tuning where the one-kernel
+    evaluator is); returns a dict of the choice."""
     g = cgeom(geom)
     n = params.shape[0] if params.dim() == 2 else params.numel() // NPAR
     t = CTuning()
@@ -519,8 +520,9 @@ def _tuning_dict(t, timed=False):
 
 
 def gbk_survey_autotune(geoms, params, obs_dev, chi2_scratch, workspace, stream=None):
-    """Times the survey launch shapes on gbk_survey_eval of this batch and
-    keeps the fastest for the survey; returns a dict of the choice."""
+    """Times the survey launch shapes, the untuned default among them, on
+    gbk_survey_eval of this batch and keeps the fastest for the survey (no
+    tuning where the default is); returns a dict of the choice."""
     arr = cgeoms(geoms)
     ws_bytes = workspace.numel() * workspace.element_size()
     t = CTuning()
