@@ -92,6 +92,13 @@ struct KahanF {
         c = (t - s) - y;
         s = t;
     }
+    // The square of x, its rounding spelt out: the same bits in every kernel.
+    __device__ __forceinline__ void add_square(float x)
+    {
+        const float y = __fmaf_rn(x, x, -c), t = s + y;
+        c = (t - s) - y;
+        s = t;
+    }
 };
 
 // LSF variance dv^2 sum_j j^2 L_j (normalised taps).

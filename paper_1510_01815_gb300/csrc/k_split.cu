@@ -127,11 +127,31 @@ gbk_status launch_split(const Geom &g, int n, const double *params, const gbk_ob
     // planes are 16 bytes a spaxel, its parts 12 bytes a tile of at least 16
     // spaxels: in practice all of them)
     TileScratch sc;
-    size_t per = (size_t)0x7fffffff / ts.tiles;
+    size_t per = (size_t)0x7fffffff / ts.tiles, room = L.pl_bytes;
+    char *scratch = (char *)ws + L.pl_off;
+    // A small batch in the shape that chi2 is bound to leaves SMs idle: where
+    // the batch's own shape (its size rounded up to a power of two: fits call
+    // with all sizes, and the shapes are remembered) is estimated at 1 / 1.7 of
+    // the cost, the residuals come in that shape and are summed afterwards (a
+    // launch of 6 - 9 us).
+    TileShape own;
+    const size_t np = (size_t)g.nx * g.ny, rbytes = resid ? 0 : al256(2 * np * sizeof(float) * (size_t)n);
+    bool two = false;
+    if (chi2 && (size_t)n * ts.tiles < 304 &&
+        rbytes + (size_t)n * (ts.tiles * sizeof(double) + sizeof(unsigned)) <= room) {
+        int m = 1;
+        while (m < n) m *= 2;
+        two = tile_shape(g, m, false, &own) && tile_cost(g, ts, m) > 1.7 * own.cost;
+    }
+    float *sums = resid;
+    if (two && !resid) {
+        sums = (float *)scratch;
+        scratch += rbytes;
+        room -= rbytes;
+    }
     if (timer && (e = timer->mark(st)) != cudaSuccess) return cuda_fail(e, "split evaluator: timing event");
     if (chi2 && ts.tiles > 1) {
-        char *scratch = (char *)ws + L.pl_off;
-        per = std::min(per, L.pl_bytes / ((size_t)ts.tiles * sizeof(double) + sizeof(unsigned)));
+        per = std::min(per, room / ((size_t)ts.tiles * sizeof(double) + sizeof(unsigned)));
         per = std::min(per, (size_t)n);
         sc.part = (double *)scratch;
         sc.arrived = (unsigned *)(scratch + per * ts.tiles * sizeof(double));
@@ -139,8 +159,12 @@ gbk_status launch_split(const Geom &g, int n, const double *params, const gbk_ob
         if (e != cudaSuccess) return cuda_fail(e, "split evaluator: clearing the arrival counters");
     }
     if (timer && (e = timer->mark(st)) != cudaSuccess) return cuda_fail(e, "split evaluator: timing event");
-    const size_t np = (size_t)g.nx * g.ny;
-    for (size_t m0 = 0; m0 < (size_t)n; m0 += per) {
+    if (two) {
+        gbk_status s = launch_tile(g, own, n, params, obs, maps, nullptr, sums, TileScratch(), batch, 0, st);
+        if (s || (s = launch_tile_resid_sum(g, ts, n, params, sums, chi2, sc, batch, 0, st))) return s;
+        if (timer) timer->launches += 2;
+    }
+    for (size_t m0 = 0; m0 < (size_t)n && !two; m0 += per) {
         const gbk_status s =
             launch_tile(g, ts, (int)std::min(per, (size_t)n - m0), params + m0 * GBK_NPAR, obs,
                         maps ? maps + 3 * np * m0 : nullptr, chi2 ? chi2 + m0 : nullptr,

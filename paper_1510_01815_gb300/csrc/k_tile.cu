@@ -436,8 +436,8 @@ __device__ __forceinline__ float y_phase(const TileItem &M, uint32_t taps, const
                         rv[h] = __ldg(M.ob.w_v + pix + h) * (m1[h] - __ldg(M.ob.v_obs + pix + h));
                         rs[h] = __ldg(M.ob.w_s + pix + h) * (m2[h] - __ldg(M.ob.s_obs + pix + h));
                     }
-                    acc.add(rv[h] * rv[h]);
-                    acc.add(rs[h] * rs[h]);
+                    acc.add_square(rv[h]);
+                    acc.add_square(rs[h]);
                 }
                 if (resid) {
                     store_pair(resid + po, rv, two, vec);
@@ -466,6 +466,28 @@ __device__ __forceinline__ double block_chi2(float v, double *red, int tid, int 
     if (tid == 0)
         for (int k = 0; k < (nthr >> 5); ++k) sum += red[k];
     return sum;
+}
+
+// A tile's part of its model's chi2 (one thread of the block): the last of a
+// model's tiles adds up all parts in tile order.
+__device__ __forceinline__ void chi2_part(double sum, bool valid, int model, int tile, int tiles, double *chi2,
+                                          double *part, unsigned *arrived)
+{
+    const double bad = (double)__int_as_float(0x7fc00000);
+    if (tiles == 1) {
+        chi2[model] = valid ? sum : bad;
+        return;
+    }
+    part[(size_t)model * tiles + tile] = sum;
+    __threadfence();
+    if (atomicAdd(&arrived[model], 1u) == (unsigned)tiles - 1) {
+        __threadfence();
+        const volatile double *p = part + (size_t)model * tiles;
+        double tot = 0.0;
+        for (int k = 0; k < tiles; ++k) tot += p[k];
+        chi2[model] = valid ? tot : bad;
+        arrived[model] = 0u;  // ready for the next call
+    }
 }
 
 // A geometry's taps, in shared memory.
@@ -583,24 +605,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) tile_kernel(const __grid_cons
         const float v = y_phase<R>(M, taps, pl, g.nx, np, a.maps, a.resid, want_obs, a.vec, tid, nthr);
         if (want_chi2) {
             const double sum = block_chi2(v, red, tid, nthr);
-            if (tid == 0) {
-                const int model = M.d.model;
-                const double bad = (double)__int_as_float(0x7fc00000);
-                if (!MULTI) {
-                    a.chi2[model] = M.mc.valid ? sum : bad;
-                } else {
-                    a.part[(size_t)model * a.tiles + M.d.tile] = sum;
-                    __threadfence();
-                    if (atomicAdd(&a.arrived[model], 1u) == (unsigned)a.tiles - 1) {
-                        __threadfence();
-                        const volatile double *p = a.part + (size_t)model * a.tiles;
-                        double tot = 0.0;
-                        for (int k = 0; k < a.tiles; ++k) tot += p[k];
-                        a.chi2[model] = M.mc.valid ? tot : bad;
-                        a.arrived[model] = 0u;  // ready for the next call
-                    }
-                }
-            }
+            if (tid == 0) chi2_part(sum, M.mc.valid, M.d.model, M.d.tile, tiles, a.chi2, a.part, a.arrived);
         }
         __syncthreads();  // the planes and the item slots change hands
         it = nxt;
@@ -612,6 +617,62 @@ __global__ void __launch_bounds__(kTileThreads, 2) tile_kernel(const __grid_cons
             buf ^= 1;
         }
     }
+}
+
+// chi2 from residuals, in the order in which tile_kernel adds them up in a
+// given shape (a CTA per tile, its threads).  Calls with chi2 are bound to the
+// shape of a large batch (TileShape); a small batch of large images leaves
+// most SMs idle in it, so it takes the residuals in a shape of its own and then
+// their sum here.  1 to 16 models of 128 x 128 x 64: 35 - 41 us in the large
+// batch's shape, 24 - 29 us so.
+struct ResidSumArgs {
+    Geom g;
+    const double *params;
+    const float *resid;      // [n][2][ny][nx]
+    const int32_t *skip;     // as TileArgs
+    int m0, mpg;
+    double *chi2, *part;
+    unsigned *arrived;
+    int tx, ty, tiles_x, tiles;
+};
+
+__global__ void __launch_bounds__(kTileThreads) tile_resid_sum_kernel(const ResidSumArgs a)
+{
+    __shared__ double red[kTileThreads / 32];
+    const int model = blockIdx.x / a.tiles, tile = blockIdx.x - model * a.tiles;
+    if (a.skip && a.skip[(a.m0 + model) / a.mpg] != 0) return;
+    const int tid = threadIdx.x, nthr = blockDim.x, nx = a.g.nx;
+    const size_t np = (size_t)nx * a.g.ny;
+    const TileDims d = tile_dims(a.g, 0, a.tx, a.ty, a.tiles_x, model, tile);
+    const float *r = a.resid + 2 * (size_t)model * np + (size_t)d.ty0 * nx + d.tx0;
+    KahanF acc;
+    const int nyq = (d.npy + 1) >> 1;
+    for (int t = tid; t < nyq * d.npx; t += nthr) {  // y_phase's tasks and their order
+        const int yq = t / d.npx, x = 2 * (t - yq * d.npx);
+        float v[2 * kNO][2];
+#pragma unroll
+        for (int o = 0; o < kNO; ++o)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const bool in = 4 * yq + o < d.nyo && x + h < d.nxo;
+                const float *q = r + (size_t)(4 * yq + o) * nx + x + h;
+                v[2 * o + h][0] = in ? q[0] : 0.f;
+                v[2 * o + h][1] = in ? q[np] : 0.f;
+            }
+#pragma unroll
+        for (int o = 0; o < kNO; ++o) {
+            if (4 * yq + o >= d.nyo) break;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                acc.add_square(v[2 * o + h][0]);
+                acc.add_square(v[2 * o + h][1]);
+            }
+        }
+    }
+    const double sum = block_chi2(acc.s - acc.c, red, tid, nthr);
+    if (tid != 0) return;
+    const bool valid = model_const(a.params + (size_t)model * GBK_NPAR, a.g).valid;
+    chi2_part(sum, valid, model, tile, a.tiles, a.chi2, a.part, a.arrived);
 }
 
 // Ragged batches: one galaxy's geometry per item, every image whole in one
@@ -720,6 +781,23 @@ static int tile_per_sm(size_t smem, int threads)
     return (int)std::min<size_t>(227 * 1024 / (smem + 3072), 800 / threads);
 }
 
+// Whole rounds of the CTA's threads: about 280 instructions a line task (two
+// spaxels), 440 an x task and 740 a y task (eight outputs), 1500 of barriers
+// and set-up.  An SM issues faster the more warps it holds, levelling off near
+// 24.
+double tile_cost(const Geom &g, const TileShape &s, int n_models)
+{
+    const double exw = s.tx + 2 * g.R, eyh = s.ty + 2 * g.R, nt = s.threads;
+    const int per_sm = tile_per_sm(s.smem, s.threads);
+    const double r1 = ceil(exw * eyh / 2 / nt), r2 = ceil(eyh / 2 * (s.tx / 4) / nt),
+                 r3 = ceil((double)s.tx / 2 * (s.ty / 4) / nt);
+    const double cta = 1500.0 + 280.0 * r1 + 440.0 * r2 + 740.0 * r3;
+    const double ctas = (double)s.tiles * n_models;
+    const double rounds = ceil(ctas / (152.0 * per_sm));
+    const double warps = std::min(ceil(ctas / 152.0), (double)per_sm) * nt / 32;
+    return rounds * cta * (10.0 + warps);
+}
+
 // The shapes of recent calls of this thread (the search takes longer than a
 // small call's kernel).
 struct ShapeKey {
@@ -756,22 +834,11 @@ bool tile_shape(const Geom &g, int n_models, bool whole, TileShape *out)
             s.tiles = s.tiles_x * ((g.ny + s.ty - 1) / s.ty);
             s.smem = tile_smem(g, s.tx, s.ty);
             if (s.smem > (size_t)kTileMaxSmem) continue;
-            const double exw = s.tx + 2 * g.R, eyh = s.ty + 2 * g.R;
             for (int nt = 128; nt <= kTileThreads; nt += 64) {
                 const int per_sm = tile_per_sm(s.smem, nt);
                 if (per_sm < 1 || (whole && per_sm < 2)) continue;
                 s.threads = nt;
-                // Whole rounds of the CTA's threads: about 280 instructions a
-                // line task (two spaxels), 440 an x task and 740 a y task
-                // (eight outputs), 1500 of barriers and set-up.  An SM issues
-                // faster the more warps it holds, levelling off near 24.
-                const double r1 = ceil(exw * eyh / 2 / nt), r2 = ceil(eyh / 2 * (s.tx / 4) / nt),
-                             r3 = ceil((double)s.tx / 2 * (s.ty / 4) / nt);
-                const double cta = 1500.0 + 280.0 * r1 + 440.0 * r2 + 740.0 * r3;
-                const double ctas = (double)s.tiles * n_models;
-                const double rounds = ceil(ctas / (152.0 * per_sm));
-                const double warps = std::min(ceil(ctas / 152.0), (double)per_sm) * nt / 32;
-                s.cost = rounds * cta * (10.0 + warps);
+                s.cost = tile_cost(g, s, n_models);
                 if (best.tiles == 0 || s.cost < best.cost) best = s;
             }
         }
@@ -838,6 +905,30 @@ gbk_status launch_tile(const Geom &g, const TileShape &ts, int n, const double *
     case 8: return launch_r<8>(a, ts, st);
     default: return fail(GBK_EUNSUPPORTED, "tile evaluator: PSF radius %d > %d", g.R, kTileMaxR);
     }
+}
+
+gbk_status launch_tile_resid_sum(const Geom &g, const TileShape &ts, int n, const double *params, const float *resid,
+                                 double *chi2, const TileScratch &scratch, const SplitBatch *batch, int m0,
+                                 cudaStream_t st)
+{
+    ResidSumArgs a = {};
+    a.g = g;
+    a.params = params;
+    a.resid = resid;
+    a.skip = batch ? batch->skip : nullptr;
+    a.m0 = m0;
+    a.mpg = batch ? batch->mpg : 1;
+    a.chi2 = chi2;
+    a.part = scratch.part;
+    a.arrived = scratch.arrived;
+    a.tx = ts.tx;
+    a.ty = ts.ty;
+    a.tiles_x = ts.tiles_x;
+    a.tiles = ts.tiles;
+    tile_resid_sum_kernel<<<n * ts.tiles, ts.threads, 0, st>>>(a);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_fail(e, "sum of residuals launch");
+    return GBK_OK;
 }
 
 // The CTA size for an image held whole, by the CTAs its planes let share an

@@ -19,14 +19,18 @@ struct TileShape {
 
 // chi2 is summed by tiles and threads, so its rounding depends on the shape:
 // every call that returns chi2 takes the shape of a batch of this many models,
-// whatever its own count.  (A fit compares a model's chi2 from batches of
-// different sizes; with equal parameters they must be equal to the bit.)
+// whatever its own count, or sums up in that order.  (A fit compares a model's
+// chi2 from batches of different sizes; with equal parameters they must be
+// equal to the bit.)
 constexpr int kTileChi2Batch = 2048;
 
 // The cheapest shape for n_models models (`whole`: one tile per model, two
 // CTAs or more per SM); false where the kernel does not serve the geometry or
 // no such shape fits.
 bool tile_shape(const Geom &g, int n_models, bool whole, TileShape *out);
+
+// A shape's estimated cost for n_models models.
+double tile_cost(const Geom &g, const TileShape &s, int n_models);
 
 // chi2 parts of `tiles` tiles per model: doubles, then arrival counters
 // (zero at the start and left zero).  Not needed for one tile per model.
@@ -39,6 +43,12 @@ struct TileScratch {
 gbk_status launch_tile(const Geom &g, const TileShape &ts, int n, const double *params, const gbk_obs *obs,
                        float *maps, double *chi2, float *resid, const TileScratch &scratch, const SplitBatch *batch,
                        int m0, cudaStream_t st);
+
+// chi2 of n models from their residuals [n][2][ny][nx], with the bits that
+// launch_tile gives in shape ts.
+gbk_status launch_tile_resid_sum(const Geom &g, const TileShape &ts, int n, const double *params, const float *resid,
+                                 double *chi2, const TileScratch &scratch, const SplitBatch *batch, int m0,
+                                 cudaStream_t st);
 
 // A ragged batch's galaxies, every image whole in one CTA.
 // Models gal * mpg + s (s < mpg) of the galaxies order[0 .. items / mpg);
