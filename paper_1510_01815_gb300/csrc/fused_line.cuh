@@ -171,10 +171,10 @@ __device__ __forceinline__ LineCtx line_ctx(const Geom &g, const ModelConst &c, 
 }
 
 // Line-of-sight velocity (Eq. 8) and surface brightness (Eq. 5) at sky
-// position (x, y), as los() in gbk_internal.cuh but with one reciprocal
+// position (x, y), as line_at() in k_staged.h but with one reciprocal
 // square root in place of the square root and the division by r, and the
 // exponential as a power of two: [Vrot(r)/r] x_e = (2/pi) Vmax atan(r/r_t)
-// (1/r) x_e with the r -> 0 limit (2/pi) Vmax / r_t.  Agrees with los() to a
+// (1/r) x_e with the r -> 0 limit (2/pi) Vmax / r_t.  Agrees with it to a
 // few FP32 ulps.
 __device__ __forceinline__ void los_line(const ModelConst &c, float x, float y, float &v, float &bright)
 {

@@ -136,21 +136,6 @@ __device__ inline ModelConst model_const(const double *p, const Geom &g)
     return c;
 }
 
-// Line-of-sight velocity (Eq. 8) and surface brightness (Eq. 5) at sky
-// position (x, y) in data pixels.  Vrot(r) cos(theta) is computed as
-// [Vrot(r)/r] x_e (Eqs. 4, 6), whose r -> 0 limit is (2/pi) Vmax / r_t.
-__device__ __forceinline__ void los(const ModelConst &c, float x, float y, float &v, float &bright)
-{
-    float dx = x - c.x0, dy = y - c.y0;
-    float xe = -dx * c.sin_pa + dy * c.cos_pa;  // Eq. 1
-    float ye = -dx * c.cos_pa - dy * c.sin_pa;  // Eq. 2
-    float yd = ye * c.inv_cos_i;
-    float r = sqrtf(xe * xe + yd * yd);         // Eq. 3
-    float f = (r > 0.f) ? c.vrot_k * atanf(r * c.inv_rt) / r : c.vrot_k * c.inv_rt;
-    v = c.vsys + f * xe * c.sin_i;              // Eq. 8
-    bright = c.i0 * expf(-r * c.inv_h);         // Eq. 5
-}
-
 // Unnormalised Gaussian tap exp(-j^2 / (2 sigma^2)) (sigma > 0).
 __device__ __forceinline__ float gauss_tap(int j, float sigma)
 {

@@ -26,9 +26,11 @@ struct StagedArgs {
     gbk_obs obs;
 };
 
-// los() with every rounding spelt out: the staged chain and the one-kernel
-// cubes get the same bits whatever the compiler would contract around the
-// call (a call that is not inlined does that too, at 2 % of the chain's time).
+// Line-of-sight velocity (Eq. 8; Vrot(r) cos(theta) as [Vrot(r) / r] x_e, Eqs.
+// 4 and 6, whose r -> 0 limit is (2/pi) Vmax / r_t) and surface brightness (Eq.
+// 5) at sky position (x, y) in data pixels, every rounding spelt out: the
+// staged chain and the one-kernel cubes get the same bits whatever the
+// compiler would contract around the call (a call that is not inlined does that too, at 2 % of the chain's time).
 static __device__ __forceinline__ float2 line_at(const ModelConst &c, float x, float y)
 {
     const float dx = __fsub_rn(x, c.x0), dy = __fsub_rn(y, c.y0);
