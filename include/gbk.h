@@ -128,8 +128,10 @@ typedef struct gbk_obs {
 /* Evaluation paths (the `flags` argument of gbk_chi2).  All compute the
  * same maps and chi-squared (Sec. 2.2.2-2.2.6); they differ in where the
  * intermediate values live.
- *  GBK_PATH_FUSED   one kernel, a thread-block cluster per model; the cube
- *                   never leaves the SM; needs no workspace.
+ *  GBK_PATH_FUSED   one kernel without a workspace, the cube never leaves the
+ *                   SM: the split path's kernel where it can (maps, and chi2
+ *                   of images that fit one CTA), else a thread-block cluster
+ *                   per model.
  *  GBK_PATH_STAGED  model cube -> separable convolution -> moments, each
  *                   stage through HBM (the paper's pipeline).
  *  GBK_PATH_SPLIT   one kernel, a CTA per model or tile of its image: each

@@ -92,7 +92,7 @@ struct GridLayout {
 };
 
 // split_bytes: the split evaluator's workspace for a chunk (0 where it does
-// not serve the geometry; the cluster evaluator then takes the chunks).
+// not serve the geometry; the fused path then takes the chunks).
 static GridLayout grid_layout(int chunk, long long nchunks, size_t split_bytes)
 {
     GridLayout L;

@@ -20,7 +20,7 @@ extern "C" gbk_status gbk_jacobian(const gbk_geom *gin, int32_t n_models, const 
     a.np = 0;
     for (int k = 0; k < GBK_NPAR; ++k)
         if (free_mask & (1u << k)) a.free_idx[a.np++] = k;
-    // velocity fields: one CTA per model, no shared-memory records
+    // velocity fields have a kernel of their own (k_vfield.cu)
     if (g.model == GBK_MODEL_CUBE && !tangent_config(g, &a.cs, &a.band, &a.direct, tangent_narrow(a)))
         return fail(GBK_EUNSUPPORTED, "geometry %d x %d too large for the Jacobian kernel", g.nx, g.ny);
     if (n_models == 0) return ok();

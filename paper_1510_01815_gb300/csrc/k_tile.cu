@@ -28,6 +28,11 @@
 // next model while the others are in the y pass.  Where an image is cut into
 // tiles the last CTA of a model (an arrival counter, reset by it) adds their
 // chi2 parts in tile order.
+//
+// What bounds it: issue slots (51 % busy) and shared-memory wavefronts (60 %).
+// Two CTAs of 384 threads an SM leave 80 registers a thread, and no instance
+// fits them: 136 - 276 bytes a thread go to local memory and 160 - 408 come
+// back, most of them around the PSF passes.
 #include <algorithm>
 
 #include "gbk_api_internal.h"
@@ -196,7 +201,7 @@ __device__ __forceinline__ void shift_sums2(f32x2 delta, f32x2 s0, f32x2 &s1, f3
     s1 = t;
 }
 
-// A tap, read where it is used: held in registers the taps would spill.
+// A tap, read where it is used: held in registers all taps would spill too.
 __device__ __forceinline__ f32x2 lds_tap(uint32_t addr)
 {
     f32x2 w;

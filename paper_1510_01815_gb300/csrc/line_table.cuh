@@ -51,8 +51,8 @@ constexpr float kLtReach = 3.0f;        // line widths served beyond the data ba
 constexpr float kLtNarrow = 0.25f;      // narrowest line served by polynomials, in channels
 constexpr float kLcNarrow = 0.45f;      // narrowest line served in closed form, in channels
 constexpr float kLcSmooth = 1.15f;      // from here on the closed form has no ripple: 2 q = 9e-12
-constexpr float kLcWindow = 6.0f;       // a line's half window for the closed form: the tails
-                                        // beyond hold 2e-9 of q0 and 4e-8 of q2
+constexpr float kLcWindow = 6.0f;       // a line's half window for the closed form: the two
+                                        // tails beyond hold 2e-9 of q0 and 7.5e-8 of q2
 
 struct LineTab {
     int nseg;            // polynomial segments stored (0: none)

@@ -10,9 +10,9 @@
 // directly;
 // all on the device; it is captured once in a CUDA graph and replayed, and
 // the host reads the number of running galaxies every kPoll iterations.  The
-// evaluations and the analytic Jacobian take the two-stage (split) kernels
-// where they serve the geometry and the caller's path allows, else the
-// one-cluster-per-model kernels; chi2 values that accept/reject compares
+// evaluations take the one-kernel evaluator and the analytic Jacobian the
+// two-stage kernels where they serve the geometry and the caller's path allows,
+// else the one-cluster-per-model kernels; chi2 values that accept/reject compares
 // always come from one evaluator.
 //
 // Plain mode: the paper's arrangement -- one galaxy at a time, the model
@@ -882,7 +882,7 @@ gbk_status lm_survey(SurveyPlan &sp, const gbk_geom *geoms, const gbk_obs *obs, 
     }
     if (pl.tangent && o->path != (int32_t)GBK_PATH_FUSED) {
         // every galaxy on the ragged split Jacobian where it serves the batch
-        // (the trial points on the survey's cluster evaluator)
+        // (the trial points on the survey's evaluator)
         TsRaggedPlan rp;
         tsplit_ragged_plan(sp.geo, &rp);
         if (rp.ok) {

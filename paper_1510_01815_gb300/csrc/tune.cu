@@ -52,7 +52,8 @@ bool fused_config_valid(const Geom &g, int cs, int threads, int persistent, Fuse
 {
     if (persistent != 0 && persistent != 1) return false;
     if (g.model != GBK_MODEL_CUBE) {
-        // the velocity-field kernel has one launch shape (one CTA per model)
+        // velocity fields choose their launch shape themselves (k_vfield.cu);
+        // this one value stands for it
         if (cs != 1 || threads != 256 || persistent != 0) return false;
         *cfg = FusedConfig{1, g.ey, 256, 0};
         return true;
