@@ -266,46 +266,21 @@ __device__ __forceinline__ void psf_pass(const Load &load, uint32_t taps, f32x2 
     }
 }
 
-// The lines of the extended tile; task: column x of a row pair, two spaxels.
-// Spaxels that neither form serves are marked with NaN and their threads come
-// back to them in a loop of their own for the direct sum: as a call from the
-// first loop it cost every model registers, and warps that took it for single
-// lanes up to half of the models' time where all lines lie outside the band.
-// Each lane of it has its own channel window; shared by the lanes that happen
-// to be there, it made the last bits depend on the tiling.
-__device__ __forceinline__ void lines_phase(const Geom &g, const TileItem &M, int R, const float *edge,
-                                            const float *ltab, float *pl, int tid, int nthr)
+// The direct sums of the spaxels that lines_phase left (marked with NaN; every
+// one where no form serves the model).  Each lane has its own channel window;
+// shared by the lanes that happen to be there, it made the last bits depend on
+// the tiling.  Out of line: beside the other phases its code costs models that
+// never take it 1 % (2048 models of 32 x 32 x 64: 51.1 us, 50.7 us so).
+static __device__ __noinline__ void lines_direct(const Geom &g, const TileItem &M, int R, const float *edge, float *pl)
 {
-    const int exw = M.d.exw, PP = M.d.PP, RP = M.d.RP, ntl = M.d.nrp * exw;
-    int x0, rp0, dx, drp;
-    split_index(tid, exw, rp0, x0);
-    split_index(nthr, exw, drp, dx);
-    const float xb = (float)(M.d.tx0 - R), yb = (float)(M.d.ty0 - R);
+    const int tid = threadIdx.x, nthr = blockDim.x;
     const bool all = line_table_empty(M.lt);
-    bool left = all;
-    if (!all) {
-        const DiscConst dc = disc_const(M.mc);
-        int x = x0, rp = rp0;
-        for (int idx = tid; idx < ntl; idx += nthr) {
-            float4 q[2];
-            line_sums_pair(dc, M.lc, M.lt, ltab, xb + (float)x, yb + (float)(2 * rp), q, left);
-            float *o = pl + rp * RP + 2 * x;
-            *reinterpret_cast<float2 *>(o) = make_float2(q[0].x, q[1].x);
-            *reinterpret_cast<float2 *>(o + PP) = make_float2(q[0].y, q[1].y);
-            *reinterpret_cast<float2 *>(o + 2 * PP) = make_float2(q[0].z, q[1].z);
-            *reinterpret_cast<float2 *>(o + 3 * PP) = make_float2(q[0].w, q[1].w);
-            x += dx;
-            rp += drp;
-            if (x >= exw) {
-                x -= exw;
-                ++rp;
-            }
-        }
-    }
-    if (!left) return;
-    const int etl = edge_table_len(g);
-    const float inv_i0 = 1.f / M.mc.i0;
-    int x = x0, rp = rp0;
+    const int exw = M.d.exw, PP = M.d.PP, RP = M.d.RP, ntl = M.d.nrp * exw, etl = edge_table_len(g);
+    const float xb = (float)(M.d.tx0 - R), yb = (float)(M.d.ty0 - R), inv_i0 = 1.f / M.mc.i0;
+    int x, rp, dx, drp;
+    split_index(tid, exw, rp, x);
+    split_index(nthr, exw, drp, dx);
+#pragma unroll 1
     for (int idx = tid; idx < ntl; idx += nthr) {
         float *const o = pl + rp * RP + 2 * x;
 #pragma unroll 1
@@ -325,6 +300,41 @@ __device__ __forceinline__ void lines_phase(const Geom &g, const TileItem &M, in
             ++rp;
         }
     }
+}
+
+// The lines of the extended tile; task: column x of a row pair, two spaxels.
+// Threads come back to the spaxels that neither form serves in a loop of their
+// own: as a call from this loop the direct sum cost every model registers, and
+// where all lines take it (narrow ones) a third of the call.
+__device__ __forceinline__ void lines_phase(const Geom &g, const TileItem &M, int R, const float *edge,
+                                            const float *ltab, float *pl, int tid, int nthr)
+{
+    bool left = true;
+    if (!line_table_empty(M.lt)) {
+        const int exw = M.d.exw, PP = M.d.PP, RP = M.d.RP, ntl = M.d.nrp * exw;
+        const DiscConst dc = disc_const(M.mc);
+        int x, rp, dx, drp;
+        split_index(tid, exw, rp, x);
+        split_index(nthr, exw, drp, dx);
+        const float xb = (float)(M.d.tx0 - R), yb = (float)(M.d.ty0 - R);
+        left = false;
+        for (int idx = tid; idx < ntl; idx += nthr) {
+            float4 q[2];
+            line_sums_pair(dc, M.lc, M.lt, ltab, xb + (float)x, yb + (float)(2 * rp), q, left);
+            float *o = pl + rp * RP + 2 * x;
+            *reinterpret_cast<float2 *>(o) = make_float2(q[0].x, q[1].x);
+            *reinterpret_cast<float2 *>(o + PP) = make_float2(q[0].y, q[1].y);
+            *reinterpret_cast<float2 *>(o + 2 * PP) = make_float2(q[0].z, q[1].z);
+            *reinterpret_cast<float2 *>(o + 3 * PP) = make_float2(q[0].w, q[1].w);
+            x += dx;
+            rp += drp;
+            if (x >= exw) {
+                x -= exw;
+                ++rp;
+            }
+        }
+    }
+    if (left) lines_direct(g, M, R, edge, pl);
 }
 
 // The x pass; task: outputs 4 xq .. 4 xq + 3 of a row pair, rows in the lanes.
@@ -525,7 +535,9 @@ __device__ __forceinline__ void tile_tables(const Geom &g, int R, TileTaps &T, f
         if (lane == 0) T.var = g.dv * g.dv * (V / S);
         if (lane < W) {
             S = 0.f;
-            for (int j = 0; j < W; ++j) S += T.w[j];
+#pragma unroll
+            for (int j = 0; j < 2 * kTileMaxR + 1; ++j)
+                if (j < W) S += T.w[j];
             const float w = T.w[lane] / S;
             T.w2[lane] = pk2(w, w);
         }
