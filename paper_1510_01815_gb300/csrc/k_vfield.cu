@@ -511,6 +511,16 @@ __global__ void __launch_bounds__(kVfThreads) vfield_tangent_many_kernel(Tangent
     }
 }
 
+// The largest batch that takes a cluster per model.  `alone`: for a call whose
+// models all run.  A fit's finished ones only return (a.skip), and its long
+// tail has few running, so there the line lies higher: fits of 512 fields of
+// 256 x 256 take 18.7 ms with clusters and 24.7 without, 300 of 128 x 128 12.6
+// and 13.3, 2048 of 64 x 64 17.7 and 14.4, 4096 of 48 x 48 24.0 and 15.3.
+static long vf_cluster_models(const Geom &g, const int32_t *skip, long alone)
+{
+    return skip ? std::max(alone, (long)g.nx * g.ny / 48) : alone;
+}
+
 gbk_status launch_vfield_tangent(const TangentArgs &a, cudaStream_t st)
 {
     if (a.geoms) return fail(GBK_EUNSUPPORTED, "survey batches serve the intensity-cube model");
@@ -521,8 +531,8 @@ gbk_status launch_vfield_tangent(const TangentArgs &a, cudaStream_t st)
     // with one CTA each, 200 of them 94 against 86; 64 of 64 x 64 23 and 23, 128
     // of them 33 against 23; 200 of 256 x 256 307 against 328, 304 of them 458
     // against 329.
-    const long np = (long)a.g.nx * a.g.ny;
-    if (a.n_models > std::min<long>(np / 64, np >= 32768 ? 208 : 152))
+    if (a.n_models > vf_cluster_models(a.g, a.skip, std::min((long)a.g.nx * a.g.ny / 64,
+                                                             (long)a.g.nx * a.g.ny >= 32768 ? 208l : 152l)))
         vfield_tangent_many_kernel<<<std::min(a.n_models, 152 * 8), kVfThreads, 0, st>>>(a);
     else
         vfield_tangent_kernel<<<a.n_models * kVfRanks, kVfThreads, 0, st>>>(a);
@@ -538,8 +548,7 @@ gbk_status launch_vfield(const FusedArgs &a, cudaStream_t st)
     // as above; only chi2's terms are exchanged here: 152 fields of 64 x 64 14
     // us against 16, 200 of them 20 against 16; 200 of 128 x 128 39 against 48,
     // 304 of them 53 against 49
-    const long np = (long)a.g.nx * a.g.ny;
-    if (a.n_models > (np >= 8192 ? 300 : 152))
+    if (a.n_models > vf_cluster_models(a.g, a.skip, (long)a.g.nx * a.g.ny >= 8192 ? 300 : 152))
         vfield_many_kernel<<<std::min(a.n_models, 152 * 16), kVfThreads, 0, st>>>(a);
     else
         vfield_kernel<<<a.n_models * kVfRanks, kVfThreads, 0, st>>>(a);
